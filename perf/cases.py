@@ -80,6 +80,13 @@ def _log_int(rng, lo, hi):
     return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
 
 
+def _whole_groups(M):
+    """Whether a filter of M particles fills a power of two of threads at 1, 2 or 4 particles each:
+    the shapes that a context takes for the paper's filter and the SIR model."""
+    groups = [-(-M // (32 * ppt)) for ppt in (1, 2, 4)]
+    return any(g & (g - 1) == 0 for g in groups)
+
+
 def draw(rng):
     kind = rng.choices(["pf", "noalloc", "run", "train", "resample"], [12, 2, 3, 1, 2])[0]
     if kind == "resample":
@@ -94,6 +101,8 @@ def draw(rng):
              "N": _log_int(rng, 1, 8192), "M": _log_int(rng, 16, 1024), "T": _log_int(rng, 5, 400)}
         if model == "sir":
             c["T"] = min(c["T"], 100)
+        if kind != "noalloc" and (model == "sir" or c["paper"]) and not _whole_groups(c["M"]):
+            continue
         if kind == "noalloc":
             c["N"] = min(c["N"], 1024)
         if kind == "run":
