@@ -671,15 +671,21 @@ __global__ void obs_terms_kernel(int model, const double* y, int T, R* obs) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= T) return;
   const double v = y[t];
-  double inv = 0.0, c = 0.0;
+  double inv = 0.0, c = 0.0, inv64 = 0.0;
   if (model != MODEL_LG && v > 0.0) {  // Poisson terms (SEIR-type and SIR)
     inv = 1.0 / v;
     c = -lgamma(v + 1.0) + v * log(v) - v;
+    if (sizeof(R) == 8 && inv >= 0x1p-1000 && inv <= 0x1p1000) {  // 1/y to a 64-bit mantissa (log_pois64)
+      const uint64_t b = (uint64_t)__double_as_longlong(inv);
+      const double lo = fma(-inv, v, 1.0) * inv;  // 1/y - inv
+      const double ulps = ldexp(lo, 63 + 1023 - (int)(b >> 52));
+      inv64 = __longlong_as_double((long long)(((b << 11) | 0x8000000000000000ull) + (uint64_t)__double2ll_rn(ulps)));
+    }
   }
   obs[4 * t] = (R)v;
   obs[4 * t + 1] = (R)inv;
   obs[4 * t + 2] = (R)c;
-  obs[4 * t + 3] = (R)0;
+  obs[4 * t + 3] = (R)inv64;
 }
 
 // Parent reference after a restored state: m_par = max_i log w_i of one dataset.

@@ -17,6 +17,7 @@ size_t pf_smem_bytes(int precision, int model, int ppt, bool general, int block,
   const int fpc = block / gt;
   const int ns = model == MODEL_LG ? 1 : model == MODEL_SIR ? 2 : 4;
   const int rs = precision == SMC2_PREC_FP64 ? 8 : 4;
+  if (rs == 8 && !is_staged(ppt)) return (size_t)fpc * region64_bytes(gt * ppt, gt, ns, model == MODEL_SIR, general);
   return (size_t)fpc * region_bytes(gt * ppt, gt >> 5, ns, rs, is_staged(ppt), general);
 }
 

@@ -208,23 +208,6 @@ __device__ __forceinline__ float warp_max_redux(float v) {
   return __int_as_float(m ^ ((m >> 31) & 0x7fffffff));
 }
 
-// slots_below split for a whole warp: the float estimate decides every crossing
-// point away from an integer (slots_estimate, which flags the others), and the
-// exact 128-bit comparison (slots_exact) settles the flagged ones.
-__device__ __forceinline__ int slots_estimate(const SlotCount& sc, float Cf, bool& near) {
-  const float est = fmaf(Cf, sc.scale, -sc.off);
-  near = !(fabsf(est - rintf(est)) > sc.margin);
-  return __float2int_ru(est);  // the ceiling, in one conversion
-}
-__device__ __forceinline__ int slots_exact(const SlotCount& sc, uint64_t C, float Cf) {
-  const float est = fmaf(Cf, sc.scale, -sc.off);
-  int n = min(max((int)rintf(est), 0), sc.M - 1);
-  const uint64_t a = ((uint64_t)n << 33) + sc.U21;
-  const uint64_t lh = __umul64hi(a, sc.S), ll = a * sc.S;
-  const uint64_t rh = __umul64hi(C, sc.M33), rl = C * sc.M33;
-  return n + ((lh < rh || (lh == rh && ll < rl)) ? 1 : 0);
-}
-
 // Barrier of one filter group of T threads (group g of its CTA).  Ungrouped
 // instantiations run one group that is the whole CTA.  Grouped ones (datasets of
 // unequal width in one launch) let a warp synchronise alone, a group that fills

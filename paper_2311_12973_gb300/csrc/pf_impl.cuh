@@ -34,6 +34,7 @@
 #include "binomial.cuh"
 #include "common.cuh"
 #include "internal.h"
+#include "soft64.cuh"
 
 namespace smc2 {
 
@@ -96,7 +97,7 @@ template <typename R, int PPT>
 struct RegCap {
   static constexpr int value =
       sizeof(R) == 4 ? (PPT <= 2 ? 64 : (PPT == 4 ? 96 : (PPT == 8 ? 128 : 168)))
-                     : (PPT == 1 ? 80 : (PPT == 2 ? 96 : (PPT <= 8 ? 128 : 168)));
+                     : (PPT <= 4 ? 80 : (PPT == 8 ? 128 : 168));
   static_assert(PPT == 1 || PPT == 2 || PPT == 4 || PPT == 8 || PPT == 16, "particles per thread");
 };
 
@@ -217,6 +218,23 @@ __device__ __forceinline__ int slots_below(const SlotCount& sc, uint64_t C, floa
   return n;
 }
 
+// slots_below split for a whole warp: the float estimate decides every crossing
+// point away from an integer (slots_estimate, which flags the others), and the
+// exact 128-bit comparison (slots_exact) settles the flagged ones.
+__device__ __forceinline__ int slots_estimate(const SlotCount& sc, float Cf, bool& near) {
+  const float est = fmaf(Cf, sc.scale, -sc.off);
+  near = !(fabsf(est - rintf(est)) > sc.margin);
+  return __float2int_ru(est);  // the ceiling, in one conversion
+}
+__device__ __forceinline__ int slots_exact(const SlotCount& sc, uint64_t C, float Cf) {
+  const float est = fmaf(Cf, sc.scale, -sc.off);
+  int n = min(max((int)rintf(est), 0), sc.M - 1);
+  const uint64_t a = ((uint64_t)n << 33) + sc.U21;
+  const uint64_t lh = __umul64hi(a, sc.S), ll = a * sc.S;
+  const uint64_t rh = __umul64hi(C, sc.M33), rl = C * sc.M33;
+  return n + ((lh < rh || (lh == rh && ll < rl)) ? 1 : 0);
+}
+
 // exp in the working precision: the FP32 path uses the hardware exp2
 // approximation (relative error about 2^-22), the FP64 path the full-precision exp.
 __device__ __forceinline__ float fast_exp(float x) { return __expf(x); }
@@ -307,6 +325,188 @@ struct FilterParams<R, MODEL_SEIR> {
   }
 };
 
+// One day of the SEIR-type dynamics in FP64 instructions, for states and parameters outside
+// the range of the fixed-point form below (it recomputes the filter's constants).
+struct SeirDay {
+  double S, E, I, lam;
+};
+static __device__ __noinline__ SeirDay seir_day_fp64(SeirDay s, double log_beta, double th2, double th3,
+                                                     const PFModel& m) {
+  const double beta = exp(log_beta), kappa = exp(th2), gamma = exp(th3);
+  const double inv_npop = 1.0 / m.npop, dt = 1.0 / m.n_sub;
+  s.lam = 0.0;
+  for (int n = 0; n < m.n_sub; ++n) {
+    const double infection = beta * s.S * s.I * inv_npop;
+    const double onset = kappa * s.E;
+    const double recovery = gamma * s.I;
+    s.lam += dt * onset;
+    s.S = fmax(s.S - dt * infection, 0.0);
+    s.E = fmax(s.E + dt * (infection - onset), 0.0);
+    s.I = fmax(s.I + dt * (onset - recovery), 0.0);
+  }
+  return s;
+}
+
+// The Poisson log-pmf y (log1p(d) - d) + c_y, d = (lambda - y) / y (no cancellation between
+// y log lambda and lambda), from the observation terms (y, 1/y, c_y, 64-bit mantissa of 1/y).
+__device__ __forceinline__ double log_pois64(double lam, const Double4& ob, const Soft64Tables& T) {
+  if (!(ob.x > 0.0)) return -lam;
+  const uint64_t inv_m = s64_bits(ob.w);
+  if (inv_m != 0ull && (uint32_t)(s64_bits(lam) >> 52) - 1u < 2046u) {  // lambda > 0 normal
+    bool ok;
+    const double g = s64_log1p_minus(lam, inv_m, (int)(s64_bits(ob.y) >> 52) - 1023, T, ok);
+    if (ok) return fma(ob.x, g, ob.z);
+  }
+  const double d = (lam - ob.x) * ob.y;
+  return ob.x * (log1p(d) - d) + ob.z;
+}
+
+// max(x, 0) of a number
+__device__ __forceinline__ double clamp0(double x) { return __double_as_longlong(x) < 0 ? 0.0 : x; }
+
+// The SEIR-type model in FP64: exp(log beta), the products beta S I dt / npop and kappa dt E and
+// the sum of E in integers with 64-bit mantissas; the sums of S, I (gamma dt I inside an FMA) and
+// lambda on the FP64 pipe, 7 operations a day, so that the two pipes take about as long.  With
+// n_sub substeps of dt:
+//   S' = S - infection, E' = (E + infection) - kappa dt E, I' = (I + onset) - gamma dt I, all >= 0.
+template <>
+struct FilterParams<double, MODEL_SEIR> {
+  double srw, nkdt, ngdt, lam_floor, S0, E0, I0, lb0, th2, th3;
+  uint64_t c_m, k_m;  // mantissas of dt / npop and kappa dt
+  int c_e, k_e;       // their exponents
+  int n_sub;
+  bool tame;          // parameters inside the range of the fixed-point form
+  __device__ void load(const double* th, const PFModel& m) {
+    lb0 = th[0];
+    th2 = th[2];
+    th3 = th[3];
+    srw = exp(th[1]);
+    const double dt = 1.0 / m.n_sub, kdt = exp(th[2]) * dt, gdt = exp(th[3]) * dt;
+    nkdt = -kdt;
+    ngdt = -gdt;
+    n_sub = m.n_sub;
+    lam_floor = m.lambda_floor;
+    S0 = m.npop - m.e0 - m.i0;
+    E0 = m.e0;
+    I0 = m.i0;
+    c_m = s64_unpack(dt / m.npop, c_e);
+    k_m = s64_unpack(kdt, k_e);
+    // no product overflows or underflows within a day: npop, kappa dt and gamma dt are moderate
+    tame = m.npop > 0x1p-20 && m.npop < 0x1p60 && kdt > 0x1p-100 && kdt < 0x1p20 && gdt < 0x1p20;
+  }
+  __device__ __forceinline__ void init(double* x, double, const double*) const {
+    x[0] = S0;
+    x[1] = E0;
+    x[2] = I0;
+    x[3] = lb0;
+  }
+  __device__ __forceinline__ void propagate(double* x, double z) const { x[3] = fma(srw, z, x[3]); }
+  // E as mantissa (leading one at bit 63, or 0) and exponent
+  __device__ __forceinline__ void substep(uint64_t bc, int eb, double& S, uint64_t& mE, int& ee, double& I,
+                                          double& lam, bool first) const {
+    int es, ei;
+    const uint64_t mS = s64_unpack(S, es), mI = s64_unpack(I, ei);
+    uint64_t p = s64_mulhi(s64_mulhi(bc, mS), mI);  // beta dt / npop (Q61 in [1, 4]) S I: Q59
+    int e = eb + es + ei + 3;
+    if (!(p >> 61)) {
+      p <<= 2;
+      e -= 2;
+    }
+    if (!(p >> 62)) {
+      p <<= 1;
+      --e;
+    }
+    if (p == 0ull || e < -1000) {
+      p = 0ull;
+      e = -1000;
+    }
+    const double inf = p == 0ull ? 0.0 : s64_pack62(p, e);
+    uint64_t o = s64_mulhi(k_m, mE);  // Q62 in [1, 4)
+    int eo = k_e + ee;
+    if (o >> 63) {
+      o >>= 1;
+      ++eo;
+    }
+    if (o == 0ull || eo < -1000) {
+      o = 0ull;
+      eo = -1000;
+    }
+    const double onset = o == 0ull ? 0.0 : s64_pack62(o, eo);
+    lam = first ? onset : lam + onset;
+    S = clamp0(S - inf);
+    I = clamp0(fma(ngdt, I, I + onset));
+    // E + infection - onset, aligned to the largest of the three (Q61 of it)
+    const int em = max(max(e, eo), ee);
+    const int64_t v = (int64_t)((mE >> 2) >> min(em - ee, 63)) + (int64_t)((p >> 1) >> min(em - e, 63)) -
+                      (int64_t)((o >> 1) >> min(em - eo, 63));
+    if (v >= (1ll << 32)) {
+      const int lz = s64_clz((uint64_t)v);
+      mE = (uint64_t)v << lz;
+      ee = em + 2 - lz;
+    } else if (v > 0) {  // nearly all of it cancelled
+      const int lz = s64_clz((uint64_t)v << 32) + 32;
+      mE = (uint64_t)v << lz;
+      ee = em + 2 - lz;
+    } else {
+      mE = 0ull;
+      ee = -1000;
+    }
+  }
+  __device__ __forceinline__ double day(double* x, const PFModel& m, const Soft64Tables& T) const {
+    double lam;
+    // |log beta| < 32, E and I below 2^257
+    if (tame && (((uint32_t)(s64_bits(x[3]) >> 52)) & 0x7ffu) < 1023u + 5u &&
+        max((uint32_t)(s64_bits(x[1]) >> 32), (uint32_t)(s64_bits(x[2]) >> 32)) < 0x50000000u) {
+      int k;
+      // e^(log beta) dt / npop: Q62 in [1, 2] times Q63 in [1, 2)
+      const uint64_t bc = s64_mulhi(s64_exp_q57(s64_q57(x[3]), T, k) << 1, c_m);
+      k += c_e;
+      double S = x[0], I = x[2];
+      int ee;
+      uint64_t mE = s64_unpack(x[1], ee);
+      substep(bc, k, S, mE, ee, I, lam, true);
+      if (n_sub == 2)
+        substep(bc, k, S, mE, ee, I, lam, false);
+      else
+        for (int s = 1; s < n_sub; ++s) substep(bc, k, S, mE, ee, I, lam, false);
+      x[0] = S;
+      x[1] = mE == 0ull || ee < -1000 ? 0.0 : s64_pack62(mE >> 1, ee);
+      x[2] = I;
+    } else {
+      const SeirDay d = seir_day_fp64({x[0], x[1], x[2], 0.0}, x[3], th2, th3, m);
+      x[0] = d.S;
+      x[1] = d.E;
+      x[2] = d.I;
+      lam = d.lam;
+    }
+    // max(lambda, floor), both non-negative (a NaN gives the floor)
+    return s64_bits(lam) > s64_bits(lam_floor) && s64_bits(lam) <= 0x7ff0000000000000ull ? lam : lam_floor;
+  }
+};
+
+// The AR(1) model in FP64: three FMA-pipe operations for the log-weight (the halving of r is
+// an exponent decrement).
+template <>
+struct FilterParams<double, MODEL_LG> {
+  double phi, sx, inv_sy, c_obs;
+  __device__ void load(const double* th, const PFModel&) {
+    const double sy = exp(th[2]);
+    phi = th[0];
+    sx = exp(th[1]);
+    inv_sy = 1.0 / sy;
+    c_obs = -0.5 * kLog2Pi - th[2];
+  }
+  __device__ __forceinline__ void init(double* x, double z0, const double*) const { x[0] = z0; }
+  __device__ __forceinline__ void propagate(double* x, double z) const { x[0] = phi * x[0] + sx * z; }
+  __device__ __forceinline__ double log_obs(const double* x, const Double4& ob) const {
+    const double r = (ob.x - x[0]) * inv_sy;
+    // -r / 2 (0 for |r| < 2^-1021, whose square is 0 too)
+    const uint64_t b = s64_bits(r);
+    const double h = s64_double((b & 0x7fe0000000000000ull) ? (b ^ 0x8000000000000000ull) - 0x0010000000000000ull : 0ull);
+    return fma(r, h, c_obs);
+  }
+};
+
 // Binomial SIR model (Sec. V-A): theta = (beta, gamma), state (S, I) integers
 // held in the working precision (exact below 2^24).  Each day, from the previous
 // day's compartments, n(S->I) ~ Bin(S, 1 - exp(-beta I / Npop)) and
@@ -342,9 +542,10 @@ struct FilterParams<R, MODEL_SIR> {
   }
   // Poisson(y; I) as for the SEIR-type model, with a point mass at 0 when I = 0
   template <typename R4>
-  __device__ __forceinline__ R log_obs(const R* x, const R4& ob) const {
+  __device__ __forceinline__ R log_obs(const R* x, const R4& ob, const Soft64Tables& T) const {
     const R I = x[1];
     if (!(I > (R)0)) return ob.x > (R)0 ? neg_inf<R>() : (R)0;
+    if constexpr (sizeof(R) == 8) return log_pois64(I, ob, T);
     if (ob.x > (R)0) {
       const R d = (I - ob.x) * ob.y;
       return ob.x * (log1p(d) - d) + ob.z;
@@ -353,6 +554,37 @@ struct FilterParams<R, MODEL_SIR> {
   }
 };
 
+// Order-preserving integer key of a number (-inf included), and its inverse: maxima of FP64
+// values by integer comparisons, which keeps them off the FP64 pipe.
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double max_num(double a, double b) { return order_key(a) > order_key(b) ? a : b; }
+__device__ __forceinline__ float max_num(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ float warp_max_num(float v) { return warp_max(v); }
+__device__ __forceinline__ double warp_max_num(double v) {  // high words, then low words among equal high ones
+  const long long k = order_key(v);
+  const int hi = (int)(k >> 32);
+  const int mh = __reduce_max_sync(0xffffffffu, hi);
+  const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? (uint32_t)k : 0u);
+  const long long m = ((long long)mh << 32) | (long long)ml;
+  return __longlong_as_double(m ^ ((m >> 63) & 0x7fffffffffffffffll));
+}
+__device__ __forceinline__ bool is_nan(float v) { return isnan(v); }
+__device__ __forceinline__ bool is_nan(double v) {
+  return (s64_bits(v) & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
+}
+
+// floor(e^a 2^B) for a = l - max <= 0 (0 below e^-37, where the value is under one)
+__device__ __forceinline__ uint64_t quantise64(double a, int B, const Soft64Tables& T) {
+  const uint32_t hi = (uint32_t)(s64_bits(a) >> 32);
+  int k;
+  const uint64_t m = s64_exp_q57(s64_q57(a), T, k);
+  // a = 0 or -37 < a < 0; a weight set whose maximum is infinite has no valid a
+  return hi == 0u || (hi - 0x80000000u) < 0x40428000u ? m >> min(61 - B - min(k, 0), 63) : 0ull;
+}
+
 // NAMED: groups wider than a warp that share a CTA synchronise on named
 // barriers 1..15 (ptxas then reserves all 16 barriers of the CTA, which limits
 // residency to four CTAs per SM).  Otherwise a wide group is the whole CTA and
@@ -360,9 +592,10 @@ struct FilterParams<R, MODEL_SIR> {
 template <typename R, int MODEL, int PPT, bool NAMED, bool GENERAL>
 __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, int i, int g, int lt,
                                            int gt, unsigned char* region, uint2 key, uint32_t k,
-                                           int t_cap) {
+                                           int t_cap, const Soft64Tables& tab) {
   constexpr int NS = ModelDims<MODEL>::NS;
   constexpr int D = ModelDims<MODEL>::D;
+  constexpr bool F64 = sizeof(R) == 8;
   using R4 = typename R4Of<R>::type;
   const int M = J.M, T = t_cap > 0 ? min(J.T, t_cap) : J.T;
   const int Mp = gt * PPT;
@@ -413,9 +646,16 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
   for (int r = 0; r < PPT; ++r) {
     R z0 = (R)0;
     if constexpr (MODEL == MODEL_LG) {
-      R z[4];
-      normals4<R>(make_uint4((uint32_t)(lt * PPT + r), 0u, c2, counter_c3(TAG_PF_INIT, k)), key, z);
-      z0 = z[0];
+      const uint4 ctr = make_uint4((uint32_t)(lt * PPT + r), 0u, c2, counter_c3(TAG_PF_INIT, k));
+      if constexpr (F64) {
+        const uint4 w = philox4x32_10(ctr, key);
+        double z1;
+        s64_normal_pair(w.x, w.y, tab, z0, z1);
+      } else {
+        R z[4];
+        normals4<R>(ctr, key, z);
+        z0 = z[0];
+      }
     }
     fp.init(x[r], z0, th);
   }
@@ -435,7 +675,20 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
   double loglik = 0.0;  // log p^(y_{1:t}) (Eq. 8)
   for (int t = 1; t <= T; ++t) {
     const int tm = (t - 1) & 3;
-    if (MODEL != MODEL_SIR && tm == 0) {  // one Philox call per particle every four steps; normals kept in shared memory
+    if (F64 && MODEL != MODEL_SIR && tm == 0) {
+#pragma unroll 1
+      for (int r = 0; r < PPT; ++r) {  // one copy of the long integer code
+        const uint4 w = philox4x32_10(make_uint4((uint32_t)(lt * PPT + r), (uint32_t)((t - 1) >> 2), c2, c3prop), key);
+        double z0, z1;
+        s64_normal_pair(w.x, w.y, tab, z0, z1);
+        Z[lt * PPT + r] = (R)z0;
+        Z[Mp + lt * PPT + r] = (R)z1;
+        s64_normal_pair(w.z, w.w, tab, z0, z1);
+        Z[2 * Mp + lt * PPT + r] = (R)z0;
+        Z[3 * Mp + lt * PPT + r] = (R)z1;
+      }
+    }
+    if (!F64 && MODEL != MODEL_SIR && tm == 0) {  // one Philox call per particle every four steps; normals kept in shared memory
 #pragma unroll
       for (int r = 0; r < PPT; ++r) {
         R z4[4];
@@ -457,16 +710,18 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
       R l;
       if constexpr (MODEL == MODEL_SIR) {
         fp.day(x[r], (uint32_t)(lt * PPT + r), (uint32_t)t, c2, c3binom, key);
-        l = fp.log_obs(x[r], ob);
+        l = fp.log_obs(x[r], ob, tab);
       } else if constexpr (MODEL == MODEL_LG) {
         fp.propagate(x[r], Z[tm * Mp + lt * PPT + r]);
         l = fp.log_obs(x[r], ob);
       } else {
         fp.propagate(x[r], Z[tm * Mp + lt * PPT + r]);
-        const R lam = fp.day(x[r]);
-        l = fp.log_pois(lam, ob);
+        if constexpr (F64)
+          l = log_pois64(fp.day(x[r], mdl, tab), ob, tab);
+        else
+          l = fp.log_pois(fp.day(x[r]), ob);
       }
-      if (isnan(l) || lt * PPT + r >= M) l = neg_inf<R>();
+      if (is_nan(l) || lt * PPT + r >= M) l = neg_inf<R>();
       if constexpr (STAGED) {
         Lw[lt * PPT + r] = l;
       } else {
@@ -474,15 +729,15 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
         ell[r] = l;
         StateVec<R, NS>::store(Xo, lt * PPT + r, x[r]);
       }
-      lmax = fmax(lmax, l);
+      lmax = max_num(lmax, l);
     }
     // (3) group maximum
-    lmax = warp_max(lmax);
+    lmax = warp_max_num(lmax);
     if (nw > 1 && lane == 0) wmax[warp] = lmax;
     group_sync();
-    if (nw > 1) lmax = warp_max(lane < nw ? wmax[lane] : neg_inf<R>());
+    if (nw > 1) lmax = warp_max_num(lane < nw ? wmax[lane] : neg_inf<R>());
     const R m = lmax;
-    if (!(m > neg_inf<R>())) {  // every weight vanished: the estimate is zero
+    if (m == neg_inf<R>()) {  // every weight vanished: the estimate is zero
       loglik = -HUGE_VAL;
       if (lt == 0 && J.delta)
         for (int s = t; s <= T; ++s) J.delta[(size_t)i * T + (s - 1)] = -HUGE_VAL;
@@ -495,7 +750,10 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
 #pragma unroll
       for (int r = 0; r < PPT; ++r) {
         const R l = Lw[lt * PPT + r];
-        run += (l > neg_inf<R>()) ? to_u64_rz(fast_exp(l - m) * scaleB) : 0ull;
+        if constexpr (F64)
+          run += quantise64(l - m, B, tab);
+        else
+          run += (l > neg_inf<R>()) ? to_u64_rz(fast_exp(l - m) * scaleB) : 0ull;
         P[lt * PPT + r] = run;
         StateVec<R, NS>::store(X, lt * PPT + r, x[r]);
       }
@@ -509,8 +767,8 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
         const R v = (ell[r] > neg_inf<R>()) ? fast_exp(ell[r] - m) * scaleB : (R)0;
         run += to_u64_rz(v);
         runf += (float)v;
-        c[r] = run;
         cf[r] = runf;
+        c[r] = run;
       }
     }
     const uint64_t incl = warp_incl_scan_u64(run, lane);
@@ -568,23 +826,17 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
       if (J.delta) J.delta[(size_t)i * T + (t - 1)] = delta;
     }
     // the schedule: every step, or when the ESS of the integer weights (Eq. 12) is below
-    // pf_ess_frac M, formed with the same correctly rounded operations as the oracle (by
-    // lane 0 of every warp, from the same totals, so the whole group decides alike)
+    // pf_ess_frac M (by lane 0 of every warp, from the same totals, so the whole group decides alike)
     bool resample = t < T;
     if (adaptive && resample) {
       int below = 0;
       if (lane == 0) {
         unsigned __int128 Q2 = 0;
         for (int w = 0; w < nw; ++w) Q2 += wq2[w];
-        if constexpr (sizeof(R) == 8) {  // the oracle's operations, bit for bit
-          const double q2 = (double)(uint64_t)(Q2 >> 64) * 0x1p64 + (double)(uint64_t)Q2;
-          const double ess = __ddiv_rn((double)S * (double)S, q2);
-          below = ess < mdl.pf_ess_frac * (double)M;
-        } else {  // mixed precision: the same test in float, S^2 < threshold sum q^2
-          const float q2 = fmaf(__ull2float_rn((uint64_t)(Q2 >> 64)), 0x1p64f, __ull2float_rn((uint64_t)Q2));
-          const float Sf = u64_to_float(S);
-          below = Sf * Sf < ess_thr * q2;
-        }
+        // the test of Eq. (12) in float: S^2 < threshold sum q^2
+        const float q2 = fmaf(__ull2float_rn((uint64_t)(Q2 >> 64)), 0x1p64f, __ull2float_rn((uint64_t)Q2));
+        const float Sf = u64_to_float(S);
+        below = Sf * Sf < ess_thr * q2;
       }
       resample = __shfl_sync(0xffffffffu, below, 0) != 0;
     }
@@ -724,10 +976,368 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
   if (lt == 0) J.loglik[i] = loglik;
 }
 
+// The FP64 filter with up to four particles per thread (M <= 2048): pf_kernel's filter with its
+// long integer functions (soft64.cuh) in loops over the thread's particles that are not
+// unrolled, and every per-particle value in shared memory.  The loop bodies are 100 to 1000
+// instructions, so a shared load and store cost them nothing, one copy of each keeps the
+// instruction cache, and a thread holds few registers whatever its particle count: the kernel is
+// bound by latency (the FP64 pipe's and its own dependent integer chains'), which more resident
+// warps hide.  SEIR, N = 1024, M = 512, T = 100: 15.4 ms with the math library's functions and
+// states in registers (FP64 pipe 85 % busy), 3.35 ms with soft64.cuh in that form, 2.80 ms in
+// this form, 2.54 ms with E's sum and the far log-weights in integers too (issue 60 %, ALU pipe
+// 61 %, FP64 pipe 48 %); 80 registers (64: 2.61 ms, 96: 3.05 ms).
+// Per-particle arrays keep particle (or slot) s at row s % PPT, column s / PPT, so that a warp
+// reading one entry per thread touches consecutive words:
+//   X    2 x [NS][Mp] double  states: step t reads buffer (t - 1) & 1 through the ancestors and
+//                             writes the other, so no copy and no barrier lies between
+//   Z    [4][Mp] double       the normals of four steps; a step's row then holds its log-weights
+//                             and quantised weights (LG and SEIR)
+//   L    [Mp] double          log-weights where they outlive the step (variants) or Z is absent (SIR)
+//   P    [Mp] u64             quantised weights of the SIR variants
+//   mark [Mp] u16, carry [T] u16   ancestors: see below
+//   wsum u64, wmax double, wq2 u128 (variants) per warp; sU u32 [8]
+// Resampling marks ancestors (Algorithm 1's order) as the FP32 filter does: particle i fills the
+// slots F(C_{i-1}) .. F(C_i) - 1; it writes its index at its first slot and as the carry of every
+// thread whose first slot it covers, and the ancestor of a slot is the largest index at or before
+// it among the thread's slots (empty marks are 0, and the reader clears them).
+template <int MODEL, bool GENERAL>
+struct Region64 {
+  static constexpr int NS = ModelDims<MODEL>::NS;
+  static constexpr bool kZ = MODEL != MODEL_SIR;
+  static constexpr bool kL = GENERAL || !kZ, kP = GENERAL && !kZ;
+};
+__host__ __device__ inline size_t region64_bytes(int Mp, int T, int ns, bool sir, bool general) {
+  size_t b = (size_t)2 * ns * Mp * 8 + (sir ? 0 : (size_t)4 * Mp * 8);
+  if (general || sir) b += (size_t)Mp * 8;
+  if (general && sir) b += (size_t)Mp * 8;
+  b += (size_t)(T >> 5) * (general ? 32 : 16) + 32;
+  b += (size_t)Mp * 2 + (size_t)T * 2;
+  return (b + 15) & ~(size_t)15;
+}
+
+template <int MODEL, int PPT, bool NAMED, bool GENERAL>
+__device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl, int i, int g, int lt, int T,
+                                             unsigned char* region, uint2 key, uint32_t k, int t_cap,
+                                             const Soft64Tables& tab) {
+  using Rg = Region64<MODEL, GENERAL>;
+  constexpr int NS = Rg::NS, D = ModelDims<MODEL>::D;
+  constexpr int LOG2P = PPT == 1 ? 0 : (PPT == 2 ? 1 : 2);
+  const int M = J.M, TT = t_cap > 0 ? min(J.T, t_cap) : J.T;
+  const int Mp = T * PPT, nw = T >> 5, lane = lt & 31, warp = lt >> 5;
+  double* X = reinterpret_cast<double*>(region);
+  double* Z = X + (size_t)2 * NS * Mp;
+  double* La = Z + (Rg::kZ ? (size_t)4 * Mp : 0);
+  uint64_t* Pa = reinterpret_cast<uint64_t*>(La + (Rg::kL ? Mp : 0));
+  unsigned __int128* wq2 = reinterpret_cast<unsigned __int128*>(Pa + (Rg::kP ? Mp : 0));  // [nw] sums of q^2
+  uint64_t* wsum = reinterpret_cast<uint64_t*>(wq2 + (GENERAL ? nw : 0));                  // [nw]
+  double* wmax = reinterpret_cast<double*>(wsum + nw);                                     // [nw]
+  uint32_t* sU = reinterpret_cast<uint32_t*>(wmax + nw);                                   // [8]
+  uint16_t* mark = reinterpret_cast<uint16_t*>(sU + 8);                                    // [Mp]
+  uint16_t* carry = mark + Mp;                                                             // [T]
+
+  auto group_sync = [&]() {
+    if (nw == 1)
+      __syncwarp();
+    else if constexpr (NAMED)
+      named_barrier(1 + g, T);
+    else
+      __syncthreads();
+  };
+
+  double th[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) th[d] = J.theta[(size_t)d * J.ld + i];
+  FilterParams<double, MODEL> fp;
+  fp.load(th, mdl);
+  const uint32_t c2 = counter_c2((uint32_t)i, J.c2hi);
+  const uint32_t c3prop = counter_c3(TAG_PF_PROP, k);
+  const uint32_t c3res = counter_c3(TAG_PF_RES, k);
+  const uint32_t c3multi = counter_c3(TAG_PF_MULTI, k);
+  const uint32_t c3binom = counter_c3(TAG_PF_BINOM, k);
+  const int B = fixed_point_bits(M);
+  const double log_norm = -(double)B * kLn2 - log((double)M);
+  const Double4* obs = reinterpret_cast<const Double4*>(J.obs);
+#pragma unroll 1
+  for (int r = 0; r < PPT; ++r) {
+    const int pos = r * T + lt;
+    double x[NS], z0 = 0.0, z1;
+    if constexpr (MODEL == MODEL_LG) {
+      const uint4 w = philox4x32_10(
+          make_uint4((uint32_t)(lt * PPT + r), 0u, c2, counter_c3(TAG_PF_INIT, k)), key);
+      s64_normal_pair(w.x, w.y, tab, z0, z1);
+    }
+    fp.init(x, z0, th);
+#pragma unroll
+    for (int e = 0; e < NS; ++e) X[(size_t)e * Mp + pos] = x[e];
+    mark[pos] = 0;
+  }
+  carry[lt] = 0;  // threads whose slots are all padding keep this valid ancestor (particle 0)
+
+  // Weights (Eq. 5): exp(Lc + l_j), Lc the common log weight set by the last resampling (Eq. 13)
+  const bool adaptive = GENERAL && mdl.pf_ess_frac > 0.0;
+  const float ess_thr = (float)(mdl.pf_ess_frac * (double)M);
+  const bool multinomial = GENERAL && mdl.pf_scheme == 1;
+  double Lc = 0.0, loglik = 0.0;  // log p^(y_{1:t}) (Eq. 8)
+  bool dead = false;
+  int from = 0;  // where the next step's states come from: 0 their own slot, 1 the marks, 2 mark[] as it stands
+  // Likelihood increments: lane (t - 1) % 32 of the group's first warp keeps step t's maximum and
+  // total, and every 32 steps the lanes take their logarithms side by side and the sum runs over
+  // them in step order (a logarithm by one lane each step would cost that warp its full time).
+  double inc_m = 0.0;
+  uint64_t inc_S = 1;
+  bool inc_res = false;
+  auto add_increments = [&](int t_last) {  // the n = (t_last - 1) % 32 + 1 steps up to t_last
+    if (warp != 0 || t_last < 1) return;
+    const int n = ((t_last - 1) & 31) + 1, t0 = t_last - n;
+    // max + log(S 2^-B) - log M, log S from its binary exponent and mantissa
+    const int e = 63 - __clzll((long long)inc_S);
+    const double mant = (double)(e >= 52 ? (inc_S >> (e - 52)) : (inc_S << (52 - e))) * 0x1p-52;
+    const double lmean = inc_m + ((double)e * kLn2 + log(mant)) + log_norm;
+    double delta = 0.0;
+    for (int s = 0; s < n; ++s) {
+      const double v = __shfl_sync(0xffffffffu, lmean, s);
+      if constexpr (GENERAL) {
+        const double logp_prev = loglik;
+        loglik = Lc + v;
+        if (lane == s) delta = loglik - logp_prev;
+        if (__shfl_sync(0xffffffffu, (int)inc_res, s)) Lc = loglik;  // Eq. (13): the mean weight from here on
+      } else {
+        loglik += v;
+        if (lane == s) delta = v;
+      }
+    }
+    if (J.delta && lane < n) J.delta[(size_t)i * TT + t0 + lane] = delta;
+  };
+
+  for (int t = 1; t <= TT; ++t) {
+    if (((t - 1) & 31) == 0) add_increments(t - 1);
+    const int tm = (t - 1) & 3;
+    const double* Xin = X + (size_t)((t - 1) & 1) * NS * Mp;
+    double* Xout = X + (size_t)(t & 1) * NS * Mp;
+    double* Lr = Rg::kL ? La : Z + (size_t)tm * Mp;
+    uint64_t* Q = Rg::kP ? Pa : (Rg::kL && !Rg::kZ ? reinterpret_cast<uint64_t*>(La)
+                                                   : reinterpret_cast<uint64_t*>(Z + (size_t)tm * Mp));
+    // (1), (2) propagate (Eq. 1) and log-weight (Eq. 2) the particles
+    uint32_t* sUg = sU + 4 * (((t - 1) >> 2) & 1);  // resampling words of four steps
+    if (tm == 0 && lt < 4 && t + lt < TT)
+      sUg[lt] = philox4x32_10(make_uint4(0u, (uint32_t)(t + lt), c2, c3res), key).x;
+    const Double4 ob = obs[t - 1];
+    double lmax = neg_inf<double>();
+    uint32_t a = carry[lt];
+#pragma unroll 1
+    for (int r = 0; r < PPT; ++r) {
+      const int j = lt * PPT + r, pos = r * T + lt;
+      if (Rg::kZ && tm == 0) {  // one Philox call every four steps
+        const uint4 w = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)((t - 1) >> 2), c2, c3prop), key);
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          double z0, z1;
+          s64_normal_pair(h ? w.z : w.x, h ? w.w : w.y, tab, z0, z1);
+          Z[(size_t)(2 * h) * Mp + pos] = z0;
+          Z[(size_t)(2 * h + 1) * Mp + pos] = z1;
+        }
+      }
+      int src = j;
+      if (!GENERAL ? t > 1 : from != 0) {
+        const uint32_t mk = mark[pos];
+        if (!GENERAL || from == 1) {
+          a = max(a, mk);
+          src = (int)a;
+          mark[pos] = 0;
+        } else {
+          src = (int)mk;
+        }
+      }
+      if (J.anc && t > 1 && j < M) J.anc[((size_t)i * (TT - 1) + (t - 2)) * M + j] = src;
+      const int spos = (src & (PPT - 1)) * T + (src >> LOG2P);
+      double x[NS], l;
+#pragma unroll
+      for (int e = 0; e < NS; ++e) x[e] = Xin[(size_t)e * Mp + spos];
+      if constexpr (MODEL == MODEL_SIR) {
+        fp.day(x, (uint32_t)j, (uint32_t)t, c2, c3binom, key);
+        l = fp.log_obs(x, ob, tab);
+      } else {
+        fp.propagate(x, Z[(size_t)tm * Mp + pos]);
+        if constexpr (MODEL == MODEL_LG)
+          l = fp.log_obs(x, ob);
+        else
+          l = log_pois64(fp.day(x, mdl, tab), ob, tab);
+      }
+#pragma unroll
+      for (int e = 0; e < NS; ++e) Xout[(size_t)e * Mp + pos] = x[e];
+      if (is_nan(l) || j >= M) l = neg_inf<double>();
+      if (adaptive && from == 0 && t > 1) l = Lr[pos] + l;  // Eq. (5) in logs: the factor since the last resampling
+      Lr[pos] = l;
+      lmax = max_num(lmax, l);
+    }
+    // (3) group maximum
+    lmax = warp_max_num(lmax);
+    if (nw > 1 && lane == 0) wmax[warp] = lmax;
+    group_sync();
+    if (nw > 1) lmax = warp_max_num(lane < nw ? wmax[lane] : neg_inf<double>());
+    const double m = lmax;
+    if (m == neg_inf<double>()) {  // every weight vanished: the estimate is zero
+      if (((t - 1) & 31) != 0) add_increments(t - 1);
+      loglik = -HUGE_VAL;
+      dead = true;
+      if (lt == 0 && J.delta)
+        for (int s = t; s <= TT; ++s) J.delta[(size_t)i * TT + (s - 1)] = -HUGE_VAL;
+      break;
+    }
+    // (4) quantise and scan
+#pragma unroll 1
+    for (int r = 0; r < PPT; ++r) Q[r * T + lt] = quantise64(Lr[r * T + lt] - m, B, tab);
+    uint64_t c[PPT];  // thread-local inclusive prefix
+    uint64_t run = 0;
+#pragma unroll
+    for (int r = 0; r < PPT; ++r) {
+      run += Q[r * T + lt];
+      c[r] = run;
+    }
+    const uint64_t incl = warp_incl_scan_u64(run, lane);
+    const uint64_t excl = incl - run;
+    if (lane == 31) wsum[warp] = incl;
+    if (adaptive) {  // the warp's sum of q^2, exact in 128 bits
+      unsigned __int128 q2 = 0;
+      uint64_t prev = 0;
+#pragma unroll
+      for (int r = 0; r < PPT; ++r) {
+        const uint64_t qv = c[r] - prev;
+        prev = c[r];
+        q2 += (unsigned __int128)qv * qv;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const uint64_t lo = __shfl_xor_sync(0xffffffffu, (uint64_t)q2, o);
+        const uint64_t hi = __shfl_xor_sync(0xffffffffu, (uint64_t)(q2 >> 64), o);
+        q2 += ((unsigned __int128)hi << 64) | lo;
+      }
+      if (lane == 0) wq2[warp] = q2;
+    }
+    group_sync();
+    // total S, and the weight `base` of the warps before this one
+    uint64_t wpre = lane < nw ? wsum[lane] : 0ull;
+    for (int o = 1; o < nw; o <<= 1) {
+      const uint64_t n = __shfl_up_sync(0xffffffffu, wpre, o);
+      if (lane >= o) wpre += n;
+    }
+    const uint64_t S = __shfl_sync(0xffffffffu, wpre, nw - 1);
+    const uint64_t base_incl = __shfl_sync(0xffffffffu, wpre, warp > 0 ? warp - 1 : 0);
+    const uint64_t C0 = (warp > 0 ? base_incl : 0ull) + excl;  // weight before the thread's first particle
+    // (5) likelihood increment (Eq. 8): see add_increments
+    const bool mine = lane == ((t - 1) & 31);
+    inc_m = mine ? m : inc_m;
+    inc_S = mine ? S : inc_S;
+    // the schedule: every step, or when the ESS of the integer weights (Eq. 12) is below
+    // pf_ess_frac M, formed with the same correctly rounded operations as the oracle (by
+    // lane 0 of every warp, from the same totals, so the whole group decides alike)
+    bool resample = t < TT;
+    if (adaptive && resample) {
+      int below = 0;
+      if (lane == 0) {
+        unsigned __int128 Q2 = 0;
+        for (int w = 0; w < nw; ++w) Q2 += wq2[w];
+        // in float first, whose error here is below 2^-20: only a near tie needs FP64
+        const float q2f = fmaf(u64_to_float((uint64_t)(Q2 >> 64)), 0x1p64f, u64_to_float((uint64_t)Q2));
+        const float Sf = u64_to_float(S), lhs = Sf * Sf, rhs = ess_thr * q2f;
+        below = lhs < rhs;
+        if (!(fabsf(lhs - rhs) > 0x1p-18f * rhs)) {
+          const double q2 = (double)(uint64_t)(Q2 >> 64) * 0x1p64 + (double)(uint64_t)Q2;
+          const double ess = __ddiv_rn((double)S * (double)S, q2);
+          below = ess < mdl.pf_ess_frac * (double)M;
+        }
+      }
+      resample = __shfl_sync(0xffffffffu, below, 0) != 0;
+    }
+    inc_res = mine ? resample : inc_res;
+    from = resample ? (multinomial ? 2 : 1) : 0;
+    if (!resample) continue;
+    if (multinomial) {
+      // slot j draws u_j = (2 U_j + 1) / 2^33 (word j & 3 of call j >> 2) and takes the
+      // first particle with C_i > floor(u_j S)
+#pragma unroll
+      for (int r = 0; r < PPT; ++r) Q[r * T + lt] = C0 + c[r];
+      group_sync();
+      uint4 wj = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int r = 0; r < PPT; ++r) {
+        const int j = lt * PPT + r;
+        if (r == 0 || (j & 3) == 0)  // a thread's consecutive slots share their calls
+          wj = philox4x32_10(make_uint4((uint32_t)j >> 2, (uint32_t)t, c2, c3multi), key);
+        if (j >= M) continue;  // padding slots keep an earlier ancestor
+        const uint32_t Uj = (j & 2) ? ((j & 1) ? wj.w : wj.z) : ((j & 1) ? wj.y : wj.x);
+        const uint64_t tau = (uint64_t)(((unsigned __int128)(2ull * Uj + 1ull) * S) >> 33);
+        int lo = 0, hi = M - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (Q[(mid & (PPT - 1)) * T + (mid >> LOG2P)] > tau)
+            hi = mid;
+          else
+            lo = mid + 1;
+        }
+        mark[r * T + lt] = (uint16_t)lo;
+      }
+      group_sync();  // Q is free: the next step may write new normals over it
+      continue;
+    }
+    // (6) systematic resampling by marks: every crossing from the float estimate, whose error is
+    // under 17 M u + 2 u (u = 2^-24: S, C0 and the thread's share reach float through two
+    // roundings each, M / S adds 4 u, the sum and the fma 1 u each, the offset 2 u absolute),
+    // covered by M 2^-19 + 2^-20; those near an integer by the exact comparison
+    SlotCount sc = slot_count_setup(sUg[tm], S, M);
+    sc.margin = fmaf((float)M, 0x1p-19f, 0x1p-20f);
+    const float C0f = u64_to_float(C0);
+    int ends[PPT + 1];
+    uint32_t near_mask = 0;
+#pragma unroll
+    for (int r = 0; r <= PPT; ++r) {
+      bool nr;
+      ends[r] = slots_estimate(sc, r == 0 ? C0f : C0f + u64_to_float(c[r - 1]), nr);
+      near_mask |= nr ? (1u << r) : 0u;
+    }
+    if (__any_sync(0xffffffffu, near_mask != 0)) {
+#pragma unroll
+      for (int r = 0; r <= PPT; ++r)
+        if (near_mask & (1u << r))
+          ends[r] = slots_exact(sc, r == 0 ? C0 : C0 + c[r - 1], r == 0 ? C0f : C0f + u64_to_float(c[r - 1]));
+    }
+#pragma unroll
+    for (int r = 0; r < PPT; ++r) {
+      const int start = ends[r], end = ends[r + 1];
+      const uint16_t id = (uint16_t)(lt * PPT + r);
+      if (end > start) mark[(start & (PPT - 1)) * T + (start >> LOG2P)] = id;
+      // the first slot of every thread inside [start, end)
+      for (int b = (start + PPT - 1) & ~(PPT - 1); b < end; b += PPT) carry[b >> LOG2P] = id;
+    }
+    group_sync();
+  }
+  if (!dead) add_increments(TT);
+  if (lt == 0) J.loglik[i] = loglik;
+  group_sync();  // the region is free for the next filter
+}
+
+// The tables of soft64.cuh as a kernel reads them: a copy in shared memory, or in the staged
+// FP64 variants, whose particles may need all of it, the device arrays.
+template <bool SHARED>
+__device__ __forceinline__ const Soft64Tables& soft64_tables() {
+  if constexpr (SHARED) {
+    __shared__ Soft64Tables s;
+    static_assert(sizeof(Soft64Tables) % 8 == 0, "copied by 8-byte words");
+    const uint64_t* from = reinterpret_cast<const uint64_t*>(&g_soft64);
+    uint64_t* to = reinterpret_cast<uint64_t*>(&s);
+    for (int w = threadIdx.x; w < (int)(sizeof(Soft64Tables) / 8); w += blockDim.x) to[w] = from[w];
+    __syncthreads();
+    return s;
+  } else {
+    return g_soft64;
+  }
+}
+
 template <typename R, int MODEL, int PPT, bool NAMED, bool GENERAL>
 __global__ void __maxnreg__((RegCap<R, PPT>::value)) pf_kernel(PFLaunch L) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_wu;
+  const Soft64Tables& tab = soft64_tables<sizeof(R) == 8 && !is_staged(PPT)>();
   constexpr int NS = ModelDims<MODEL>::NS;
   const uint32_t k = L.k_done ? (uint32_t)(*L.k_done + 1) : (uint32_t)L.k_imm;
   const uint2 key = seed_key(L.seed);
@@ -756,10 +1366,15 @@ __global__ void __maxnreg__((RegCap<R, PPT>::value)) pf_kernel(PFLaunch L) {
     const PFJob J = L.jobs ? L.jobs[job] : L.job0;
     const int gt = group_threads_for(PPT, J.M);
     const int g = threadIdx.x / gt, lt = threadIdx.x - g * gt;
-    const size_t rb = region_bytes(gt * PPT, gt >> 5, NS, (int)sizeof(R), is_staged(PPT), GENERAL);
-    if (g < count && (g + 1) * gt <= (int)blockDim.x)
-      run_filter<R, MODEL, PPT, NAMED, GENERAL>(J, L.mdl, first + g, g, lt, gt, smem + g * rb, key, k,
-                                                L.t_cap);
+    if constexpr (sizeof(R) == 8 && !is_staged(PPT)) {
+      const size_t rb = region64_bytes(gt * PPT, gt, NS, MODEL == MODEL_SIR, GENERAL);
+      if (g < count && (g + 1) * gt <= (int)blockDim.x)
+        run_filter64<MODEL, PPT, NAMED, GENERAL>(J, L.mdl, first + g, g, lt, gt, smem + g * rb, key, k, L.t_cap, tab);
+    } else {
+      const size_t rb = region_bytes(gt * PPT, gt >> 5, NS, (int)sizeof(R), is_staged(PPT), GENERAL);
+      if (g < count && (g + 1) * gt <= (int)blockDim.x)
+        run_filter<R, MODEL, PPT, NAMED, GENERAL>(J, L.mdl, first + g, g, lt, gt, smem + g * rb, key, k, L.t_cap, tab);
+    }
     if (!L.wu_counter) __syncthreads();
   }
 }
