@@ -133,12 +133,17 @@ __device__ __forceinline__ int fixed_point_bits(int n) {
   return b < 52 ? b : 52;
 }
 
-// floor((2^33 j + 2U + 1) S / (n 2^33)): the threshold of slot j.
+// floor((2^33 j + 2U + 1) S / (n 2^33)): the threshold of slot j < n < 2^15.  The shift by 33
+// comes first (floors nest), which leaves less than 2^78; the division by n then takes two steps
+// of 64 by 32 bits in place of a general 128-bit one.
 __device__ __forceinline__ uint64_t slot_threshold(uint32_t j, uint32_t U, uint64_t S, int n,
                                                    int log2n) {
   const unsigned __int128 num = (((unsigned __int128)j << 33) + 2ull * U + 1ull) * S;
   if (log2n >= 0) return (uint64_t)(num >> (33 + log2n));
-  return (uint64_t)(num / ((unsigned __int128)n << 33));
+  const unsigned __int128 a = num >> 33;
+  const uint64_t top = (uint64_t)(a >> 32), q1 = top / (uint32_t)n;
+  const uint64_t low = ((top - q1 * (uint32_t)n) << 32) | (uint32_t)a;
+  return (q1 << 32) + low / (uint32_t)n;
 }
 
 template <typename R>

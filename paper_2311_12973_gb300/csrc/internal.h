@@ -19,7 +19,7 @@
 namespace smc2 {
 
 constexpr int kOuterBlock = 32;                        // threads of the per-sample outer kernels (one warp)
-constexpr int kResBlock = 256;                         // threads of the resampling kernel
+constexpr int kResBlock = 512;                         // threads of the resampling kernel
 constexpr int kPfMaxBlock = 512;                       // threads of a particle-filter CTA, at most
 constexpr int kMlpH = 64;                              // hidden width of the surrogate network
 constexpr int kMlpWarps = 4;                           // warps (16 rows each) per network CTA
