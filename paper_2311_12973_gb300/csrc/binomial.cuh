@@ -36,10 +36,9 @@ struct BinomWords {
 
   __device__ __forceinline__ BinomWords(uint4 c, uint2 k) : ctr(c), key(k), cur(), left(0), calls(0) {}
 
-  // next uniform in (0, 1), or 0 when the stream is spent
-  __device__ __forceinline__ double next() {
+  // the next word (calls < 64 or words left)
+  __device__ __forceinline__ uint32_t word() {
     if (left == 0) {
-      if (calls == 64) return 0.0;
       cur = philox4x32_10(make_uint4(ctr.x + 4096u * (uint32_t)calls, ctr.y, ctr.z, ctr.w), key);
       ++calls;
       left = 4;
@@ -49,7 +48,12 @@ struct BinomWords {
     cur.y = cur.z;
     cur.z = cur.w;
     --left;
-    return ((double)w * 2.0 + 1.0) * 0x1p-33;  // exact
+    return w;
+  }
+  // next uniform in (0, 1), or 0 when the stream is spent
+  __device__ __forceinline__ double next() {
+    if (left == 0 && calls == 64) return 0.0;
+    return ((double)word() * 2.0 + 1.0) * 0x1p-33;  // exact
   }
 };
 
@@ -143,6 +147,110 @@ __device__ __forceinline__ float stirling_fc(float j) {
   }
   const float r = __fdividef(1.f, x), r2 = r * r;
   return r * (1.f / 12.f - r2 * (1.f / 360.f - r2 * (1.f / 1260.f)));
+}
+
+// ---------------------------------------------------------------------------
+// Bin(n, p) of the FP64 form with its decisions taken in FP32 and integers where they are clear.
+// FP64 instructions are so slow on this GPU (78 issue slots each) that the draw above takes the
+// time of thousands of others, while every decision it takes -- the regime, the inversion's
+// crossing, floor(), the squeeze and the exact test -- is a comparison that FP32 settles unless it
+// is near a tie.  Each comparison below carries a margin of at least four times its FP32 error
+// (1.2e8 draws over n to 2^24 with every margin a quarter as wide: none went wrong); inside a
+// margin ok is false and the caller draws again with the FP64 form from the same place of the
+// stream, so the result is always that form's.  At n = 1e4 about one draw in 8000 is.
+// n p, its integer part and floor((n + 1) p) come from p in fixed point, pq = p 2^63 to 2^-56.
+// n <= 2^24.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float q63_to_float(uint64_t v) {  // v 2^-63
+  return fmaf(__uint2float_rn((uint32_t)(v >> 32)), 0x1p-31f, __uint2float_rn((uint32_t)v) * 0x1p-63f);
+}
+// n v 2^-63 in Q31
+__device__ __forceinline__ uint64_t times_q63(uint32_t n, uint64_t v) {
+  return (uint64_t)n * (uint32_t)(v >> 32) + (((uint64_t)n * (uint32_t)v) >> 32);
+}
+// log1p(x) - x, x > -1: by the series of s = x / (2 + x), -s x + 2 s^3 (1/3 + s^2/5 + ...), for |s| <= 1/3
+__device__ __forceinline__ float log1p_minus_f(float x) {
+  const float s = __fdividef(x, x + 2.f), s2 = s * s;
+  float p = fmaf(s2, 1.f / 13.f, 1.f / 11.f);
+  p = fmaf(s2, p, 1.f / 9.f);
+  p = fmaf(s2, p, 1.f / 7.f);
+  p = fmaf(s2, p, 1.f / 5.f);
+  p = fmaf(s2, p, 1.f / 3.f);
+  return fabsf(s) <= 1.f / 3.f ? fmaf(-s, x, 2.f * s2 * s * p) : log1pf(x) - x;
+}
+__device__ __forceinline__ uint32_t binomial_filtered(uint32_t n, uint64_t pq, BinomWords& b, bool& ok) {
+  constexpr uint64_t kOne = 1ull << 63, kHalf = 1ull << 62, kTiny = 1ull << 23;
+  const bool flip = pq > kHalf;
+  if (flip) pq = kOne - pq;
+  const uint64_t np = times_q63(n, pq);
+  constexpr uint64_t kTen = 10ull << 31;
+  ok = pq > kTiny && pq < kHalf - kTiny && (np < kTen - 4 || np > kTen + 4);
+  const float pf = q63_to_float(pq), qf = q63_to_float(kOne - pq), nf = (float)n;
+  uint32_t k = 0;
+  if (np < kTen) {
+    // inversion: the first k with u <= P(0) + .. + P(k)
+    const float sf = __fdividef(pf, qf), a = (nf + 1.f) * sf;
+    const float u = ((float)b.word() + 0.5f) * 0x1p-32f;
+    constexpr float kMargin = 0x1p-16f;  // the sums' error is below 2^-18 for n p < 10
+    float r = __expf(nf * log1pf(-pf)), sum = r, below = -1.f, kf = 0.f;
+    while (u > sum && kf < 100.f) {
+      kf += 1.f;
+      r *= __fdividef(a, kf) - sf;
+      below = sum;
+      sum += r;
+    }
+    ok = ok && kf <= nf && u - below > kMargin && sum - u > kMargin;
+    k = (uint32_t)kf;
+  } else {
+    const uint64_t c = np + (1ull << 30);  // n p + 1/2
+    const int ci = (int)(c >> 31);
+    const float cf = (float)(uint32_t)(c & 0x7fffffffu) * 0x1p-31f;
+    const float spq = sqrtf((float)np * 0x1p-31f * qf);
+    const float bb = 1.15f + 2.53f * spq;
+    const float aa = -0.0873f + 0.0248f * bb + 0.01f * pf;
+    const float vr = 0.92f - __fdividef(4.2f, bb);
+    for (int tries = 0;; ++tries) {
+      const uint32_t w1 = b.word(), w2 = b.word();
+      const int s = (int)(w1 ^ 0x80000000u);  // u = (s + 1/2) 2^-32, us = 1/2 - |u| = (si + 1/2) 2^-32
+      const uint32_t si = s >= 0 ? 0x7fffffffu - (uint32_t)s : 0x80000000u + (uint32_t)s;
+      const float us = ((float)si + 0.5f) * 0x1p-32f;
+      const float t = (__fdividef(2.f * aa, us) + bb) * (((float)s + 0.5f) * 0x1p-32f) + cf;
+      const float fl = floorf(t), mg = fmaf(fabsf(t), 0x1p-20f, 0x1p-18f);
+      ok = ok && tries < 8;
+      if (!ok) break;
+      if (t < -(float)ci - 1.f - mg || t > (float)((int)n - ci) + 1.f + mg) continue;  // k < 0 or k > n
+      ok = t - fl > mg && t - fl < 1.f - mg;
+      const int ki = ci + (int)fl;
+      if (ok && (ki < 0 || ki > (int)n)) continue;
+      k = (uint32_t)ki;
+      const float v = ((float)w2 + 0.5f) * 0x1p-32f;
+      if (si >= 300647711u) {  // us >= 0.07
+        ok = ok && fabsf(v - vr) > 0x1p-20f;
+        if (!ok || v < vr) break;
+      }
+      if (!ok) break;
+      // the exact test: with x1 = (m - k) / (k + 1), x2 = (k - m) / (n - k + 1) and g(x) = log1p(x) - x the
+      // linear parts of the FP32 sampler's form (below) combine, and no term exceeds the result's size by much:
+      //   log f(k)/f(m) = (k - m) ((k - m + 1/2) / (k + 1) + (k - m - 1/2) / (n - k + 1))
+      //     + (m + 1/2) g(x1) + (n - m + 1/2) g(x2) + (k - m) log1p(((n + 2) p - (k + 1)) / ((k + 1) q)) + fc's
+      const uint64_t m31 = np + (pq >> 32);  // (n + 1) p
+      const uint32_t mfrac = (uint32_t)(m31 & 0x7fffffffu), mi = (uint32_t)(m31 >> 31);
+      ok = mfrac > 64u && mfrac < 0x7fffffffu - 64u;
+      const float kf = (float)k, mf = (float)mi, km = (float)(int)(k - mi);
+      const float d = (float)((long long)(np + 2 * (pq >> 32)) - ((long long)(k + 1u) << 31)) * 0x1p-31f;  // (n + 2) p - (k + 1)
+      const float rk = __fdividef(1.f, kf + 1.f), rn = __fdividef(1.f, nf - kf + 1.f);
+      const float t0 = km * ((km + 0.5f) * rk + (km - 0.5f) * rn);
+      const float t1 = (mf + 0.5f) * log1p_minus_f(-km * rk);
+      const float t2 = (nf - mf + 0.5f) * log1p_minus_f(km * rn);
+      const float t3 = km * log1pf(__fdividef(d * rk, qf));
+      const float lr = t0 + t1 + t2 + t3 + (stirling_fc(mf) + stirling_fc(nf - mf)) - stirling_fc(kf) - stirling_fc(nf - kf);
+      const float alpha = (2.83f + __fdividef(5.1f, bb)) * spq;
+      const float lv = logf(__fdividef(v * alpha, __fdividef(aa, us * us) + bb));
+      ok = ok && fabsf(lv - lr) > fmaf(t0 + fabsf(t1) + fabsf(t2) + fabsf(t3), 0x1p-19f, 0x1p-17f);
+      if (!ok || lv < lr) break;
+    }
+  }
+  return flip ? n - k : k;
 }
 
 struct BinomWordsF {

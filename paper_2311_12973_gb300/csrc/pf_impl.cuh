@@ -534,7 +534,7 @@ struct FilterParams<R, MODEL_SIR> {
     const R S = x[0], I = x[1];
     const R h = beta * I / npop;
     const R p_si = -expm1(-h);
-    typename std::conditional<sizeof(R) == 8, BinomWords, BinomWordsF>::type b(make_uint4(j, t, c2, c3), key);
+    BinomWordsF b(make_uint4(j, t, c2, c3), key);
     const R n_si = binomial_draw(S, p_si, b);
     const R n_ir = binomial_draw(I, p_ir, b);
     x[0] = S - n_si;
@@ -542,15 +542,80 @@ struct FilterParams<R, MODEL_SIR> {
   }
   // Poisson(y; I) as for the SEIR-type model, with a point mass at 0 when I = 0
   template <typename R4>
-  __device__ __forceinline__ R log_obs(const R* x, const R4& ob, const Soft64Tables& T) const {
+  __device__ __forceinline__ R log_obs(const R* x, const R4& ob, const Soft64Tables&) const {
     const R I = x[1];
     if (!(I > (R)0)) return ob.x > (R)0 ? neg_inf<R>() : (R)0;
-    if constexpr (sizeof(R) == 8) return log_pois64(I, ob, T);
     if (ob.x > (R)0) {
       const R d = (I - ob.x) * ob.y;
       return ob.x * (log1p(d) - d) + ob.z;
     }
     return -I;
+  }
+};
+
+// One flow drawn by the FP64 sampler, for the draws that binomial_filtered leaves open.
+static __device__ __noinline__ double sir_flow_fp64(double n, double p, double hazard, BinomWords& b) {
+  return binomial_draw(n, hazard != 0.0 ? -expm1(-hazard) : p, b);
+}
+
+// The same model in FP64.  The draws' decisions come from binomial_filtered, whose probability
+// for the S->I flow is 1 - e^(-beta I / npop) in fixed point; draws that it leaves open (one in
+// 8000 at npop = 1e4) run the FP64 sampler, whose results all draws have.
+// N = 256, M = 500, T = 30: 13.8 ms with every draw by the FP64 sampler (FP64 pipe 85 % busy), 0.98 ms so.
+template <>
+struct FilterParams<double, MODEL_SIR> {
+  double beta, npop, rate, S0, I0, p_ir;  // rate = beta / npop
+  uint64_t pq_ir;                         // p_ir in Q63; 0: the flow needs the FP64 sampler
+  __device__ void load(const double* th, const PFModel& m) {
+    beta = th[0];
+    npop = m.npop;
+    rate = beta / npop;
+    p_ir = -expm1(-th[1]);
+    pq_ir = p_ir > 0x1p-30 && p_ir < 1.0 - 0x1p-30 ? (uint64_t)__double2ull_rz(p_ir * 0x1p63) : 0ull;
+    S0 = m.npop - m.i0;
+    I0 = m.i0;
+  }
+  __device__ __forceinline__ void init(double* x, double, const double*) const {
+    x[0] = S0;
+    x[1] = I0;
+  }
+  __device__ __forceinline__ void day(double* x, uint32_t j, uint32_t t, uint32_t c2, uint32_t c3, uint2 key,
+                                      const Soft64Tables& T) const {
+    // compartments are integers below 2^24: their low words after adding 2^52
+    const uint32_t S = (uint32_t)s64_bits(x[0] + 0x1p52), I = (uint32_t)s64_bits(x[1] + 0x1p52);
+    const double h = x[1] * rate;
+    uint64_t pq_si = 0ull;
+    if (h > 0x1p-40 && h < 20.0) {
+      int k;
+      const uint64_t e = s64_exp_q57(s64_q57(-h), T, k);  // Q61 2^k, k < 0 (0 next to h = 0)
+      pq_si = (1ull << 63) - ((e << 2) >> min(-k, 63));
+    }
+    BinomWords b(make_uint4(j, t, c2, c3), key);
+    uint32_t flow = 0, n_si = 0;
+#pragma unroll 1
+    for (int f = 0; f < 2; ++f) {
+      const uint32_t n = f ? I : S;
+      const uint64_t pq = f ? pq_ir : pq_si;
+      n_si = flow;
+      flow = 0;
+      if (n != 0u && (f ? p_ir > 0.0 : h > 0.0)) {
+        const BinomWords start = b;
+        bool ok = false;
+        if (pq != 0ull) flow = binomial_filtered(n, pq, b, ok);
+        if (!ok) {
+          BinomWords again = start;
+          flow = (uint32_t)sir_flow_fp64((double)n, p_ir, f ? 0.0 : beta * x[1] / npop, again);
+          b = again;
+        }
+      }
+    }
+    x[0] = s64_double(0x4330000000000000ull | (S - n_si)) - 0x1p52;
+    x[1] = s64_double(0x4330000000000000ull | (I + n_si - flow)) - 0x1p52;
+  }
+  __device__ __forceinline__ double log_obs(const double* x, const Double4& ob, const Soft64Tables& T) const {
+    const double I = x[1];
+    if (!(I > 0.0)) return ob.x > 0.0 ? neg_inf<double>() : 0.0;
+    return log_pois64(I, ob, T);
   }
 };
 
@@ -1154,7 +1219,7 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
 #pragma unroll
       for (int e = 0; e < NS; ++e) x[e] = Xin[(size_t)e * Mp + spos];
       if constexpr (MODEL == MODEL_SIR) {
-        fp.day(x, (uint32_t)j, (uint32_t)t, c2, c3binom, key);
+        fp.day(x, (uint32_t)j, (uint32_t)t, c2, c3binom, key, tab);
         l = fp.log_obs(x, ob, tab);
       } else {
         fp.propagate(x, Z[(size_t)tm * Mp + pos]);
