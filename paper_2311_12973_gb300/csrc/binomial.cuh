@@ -168,7 +168,7 @@ __device__ __forceinline__ float q63_to_float(uint64_t v) {  // v 2^-63
 __device__ __forceinline__ uint64_t times_q63(uint32_t n, uint64_t v) {
   return (uint64_t)n * (uint32_t)(v >> 32) + (((uint64_t)n * (uint32_t)v) >> 32);
 }
-// log1p(x) - x, x > -1: by the series of s = x / (2 + x), -s x + 2 s^3 (1/3 + s^2/5 + ...), for |s| <= 1/3
+// log1p(x) - x, x > -1, to about 2^-21 of its terms: by the series of s = x / (2 + x), -s x + 2 s^3 (1/3 + s^2/5 + ...), for |s| <= 1/3
 __device__ __forceinline__ float log1p_minus_f(float x) {
   const float s = __fdividef(x, x + 2.f), s2 = s * s;
   float p = fmaf(s2, 1.f / 13.f, 1.f / 11.f);
@@ -176,7 +176,38 @@ __device__ __forceinline__ float log1p_minus_f(float x) {
   p = fmaf(s2, p, 1.f / 7.f);
   p = fmaf(s2, p, 1.f / 5.f);
   p = fmaf(s2, p, 1.f / 3.f);
-  return fabsf(s) <= 1.f / 3.f ? fmaf(-s, x, 2.f * s2 * s * p) : log1pf(x) - x;
+  const float series = fmaf(-s, x, 2.f * s2 * s * p);
+  if (fabsf(s) <= 1.f / 3.f) return series;
+  return __logf(1.f + x) - x;
+}
+// fc(j) of the FP32 sampler below, short form
+static __device__ const float g_stirling_fc[10] = {0.0810614668f, 0.0413406960f, 0.0276779257f, 0.0207906721f,
+                                                   0.0166446912f, 0.0138761288f, 0.0118967099f, 0.0104112653f,
+                                                   0.00925546218f, 0.00833056343f};
+__device__ __forceinline__ float stirling_fc_short(float j) {
+  if (j < 10.f) return g_stirling_fc[(int)j];
+  const float r = __fdividef(1.f, j + 1.f);
+  return r * fmaf(-r * r, 1.f / 360.f, 1.f / 12.f);  // the next term is below 1e-8
+}
+// BTRS's exact test without a tie: log f(k)/f(m) - log(v alpha / (a / us^2 + b)), with
+// d = (n + 2) p - (k + 1), x1 = (m - k) / (k + 1), x2 = (k - m) / (n - k + 1) and g(x) = log1p(x) - x from
+//   log f(k)/f(m) = (k - m) ((k - m + 1/2) / (k + 1) + (k - m - 1/2) / (n - k + 1))
+//     + (m + 1/2) g(x1) + (n - m + 1/2) g(x2) + (k - m) log1p(d / ((k + 1) q)) + fc(m) + fc(n - m) - fc(k) - fc(n - k),
+// which is the FP32 sampler's form (below) with the linear parts of its logarithms combined, so that no
+// term exceeds the result by much.  `size` receives the sum of the terms' magnitudes.
+__device__ __forceinline__ float btrs_excess(float n, float k, float m, float q, float d, float v, float us, float aa,
+                                             float bb, float spq, float& size) {
+  const float km = k - m, rk = __fdividef(1.f, k + 1.f), rn = __fdividef(1.f, n - k + 1.f);
+  const float t0 = km * ((km + 0.5f) * rk + (km - 0.5f) * rn);
+  const float t1 = (m + 0.5f) * log1p_minus_f(-km * rk);
+  const float t2 = (n - m + 0.5f) * log1p_minus_f(km * rn);
+  const float x3 = __fdividef(d * rk, q);
+  const float t3 = km * (log1p_minus_f(x3) + x3);
+  const float fc = (stirling_fc_short(m) + stirling_fc_short(n - m)) - stirling_fc_short(k) - stirling_fc_short(n - k);
+  const float alpha = (2.83f + __fdividef(5.1f, bb)) * spq;
+  const float lv = __logf(__fdividef(v * alpha, __fdividef(aa, us * us) + bb));
+  size = fabsf(t0) + fabsf(t1) + fabsf(t2) + fabsf(t3) + fabsf(lv);
+  return t0 + t1 + t2 + t3 + fc - lv;
 }
 __device__ __forceinline__ uint32_t binomial_filtered(uint32_t n, uint64_t pq, BinomWords& b, bool& ok) {
   constexpr uint64_t kOne = 1ull << 63, kHalf = 1ull << 62, kTiny = 1ull << 23;
@@ -229,25 +260,13 @@ __device__ __forceinline__ uint32_t binomial_filtered(uint32_t n, uint64_t pq, B
         if (!ok || v < vr) break;
       }
       if (!ok) break;
-      // the exact test: with x1 = (m - k) / (k + 1), x2 = (k - m) / (n - k + 1) and g(x) = log1p(x) - x the
-      // linear parts of the FP32 sampler's form (below) combine, and no term exceeds the result's size by much:
-      //   log f(k)/f(m) = (k - m) ((k - m + 1/2) / (k + 1) + (k - m - 1/2) / (n - k + 1))
-      //     + (m + 1/2) g(x1) + (n - m + 1/2) g(x2) + (k - m) log1p(((n + 2) p - (k + 1)) / ((k + 1) q)) + fc's
       const uint64_t m31 = np + (pq >> 32);  // (n + 1) p
       const uint32_t mfrac = (uint32_t)(m31 & 0x7fffffffu), mi = (uint32_t)(m31 >> 31);
-      ok = mfrac > 64u && mfrac < 0x7fffffffu - 64u;
-      const float kf = (float)k, mf = (float)mi, km = (float)(int)(k - mi);
       const float d = (float)((long long)(np + 2 * (pq >> 32)) - ((long long)(k + 1u) << 31)) * 0x1p-31f;  // (n + 2) p - (k + 1)
-      const float rk = __fdividef(1.f, kf + 1.f), rn = __fdividef(1.f, nf - kf + 1.f);
-      const float t0 = km * ((km + 0.5f) * rk + (km - 0.5f) * rn);
-      const float t1 = (mf + 0.5f) * log1p_minus_f(-km * rk);
-      const float t2 = (nf - mf + 0.5f) * log1p_minus_f(km * rn);
-      const float t3 = km * log1pf(__fdividef(d * rk, qf));
-      const float lr = t0 + t1 + t2 + t3 + (stirling_fc(mf) + stirling_fc(nf - mf)) - stirling_fc(kf) - stirling_fc(nf - kf);
-      const float alpha = (2.83f + __fdividef(5.1f, bb)) * spq;
-      const float lv = logf(__fdividef(v * alpha, __fdividef(aa, us * us) + bb));
-      ok = ok && fabsf(lv - lr) > fmaf(t0 + fabsf(t1) + fabsf(t2) + fabsf(t3), 0x1p-19f, 0x1p-17f);
-      if (!ok || lv < lr) break;
+      float size;
+      const float ex = btrs_excess(nf, (float)k, (float)mi, qf, d, v, us, aa, bb, spq, size);
+      ok = mfrac > 64u && mfrac < 0x7fffffffu - 64u && fabsf(ex) > fmaf(size, 0x1p-19f, 0x1p-17f);
+      if (!ok || ex > 0.f) break;
     }
   }
   return flip ? n - k : k;
@@ -277,6 +296,25 @@ struct BinomWordsF {
   }
 };
 
+// BTRS's exact test in float (true: accept)
+static __device__ __noinline__ bool btrs_exact_f32(float n, float p, float k, float us, float v1, float aa, float bb,
+                                                   float spq) {
+  const float q = 1.f - p;
+  const float m = floorf(fmaf(n, p, p));  // floor((n + 1) p), one rounding
+  const float fcm = stirling_fc(m) + stirling_fc(n - m);
+  const float alpha = (2.83f + __fdividef(5.1f, bb)) * spq;
+  const float n2 = n + 2.f;
+  const float np2 = n2 * p;
+  const float np2_err = fmaf(n2, p, -np2);  // (n + 2) p = np2 + np2_err exactly
+  const float d = ((np2 - (k + 1.f)) + np2_err);
+  const float lr = (m + 0.5f) * log1pf(__fdividef(m - k, k + 1.f)) +
+                   (n - m + 0.5f) * log1pf(__fdividef(k - m, n - k + 1.f)) +
+                   (k - m) * log1pf(__fdividef(d, (k + 1.f) * q)) + fcm - stirling_fc(k) -
+                   stirling_fc(n - k);
+  const float v = logf(__fdividef(v1 * alpha, __fdividef(aa, us * us) + bb));
+  return v <= lr;
+}
+
 static __device__ __noinline__ float binomial_half_f32(float n, float p, BinomWordsF& b) {
   const float q = 1.f - p;
   if (n * p < 10.f) {
@@ -302,8 +340,7 @@ static __device__ __noinline__ float binomial_half_f32(float n, float p, BinomWo
   const float c = n * p + 0.5f;
   const float ci = floorf(c), cf = c - ci;
   const float vr = 0.92f - __fdividef(4.2f, bb);
-  bool have_m = false;
-  float m = 0.f, fcm = 0.f, alpha = 0.f, np2 = 0.f, np2_err = 0.f;
+  const float m = floorf(fmaf(n, p, p));  // floor((n + 1) p), one rounding
   for (;;) {
     const float u1 = b.next();
     const float v1 = b.next();
@@ -313,22 +350,18 @@ static __device__ __noinline__ float binomial_half_f32(float n, float p, BinomWo
     const float k = ci + floorf((__fdividef(2.f * aa, us) + bb) * u + cf);
     if (k < 0.f || k > n) continue;
     if (us >= 0.07f && v1 <= vr) return k;
-    if (!have_m) {
-      m = floorf(fmaf(n, p, p));  // floor((n + 1) p), one rounding
-      fcm = stirling_fc(m) + stirling_fc(n - m);
-      alpha = (2.83f + __fdividef(5.1f, bb)) * spq;
-      const float n2 = n + 2.f;
-      np2 = n2 * p;
-      np2_err = fmaf(n2, p, -np2);  // (n + 2) p = np2 + np2_err exactly
-      have_m = true;
-    }
-    const float d = ((np2 - (k + 1.f)) + np2_err);
-    const float lr = (m + 0.5f) * log1pf(__fdividef(m - k, k + 1.f)) +
-                     (n - m + 0.5f) * log1pf(__fdividef(k - m, n - k + 1.f)) +
-                     (k - m) * log1pf(__fdividef(d, (k + 1.f) * q)) + fcm - stirling_fc(k) -
-                     stirling_fc(n - k);
-    const float v = logf(__fdividef(v1 * alpha, __fdividef(aa, us * us) + bb));
-    if (v <= lr) return k;
+    // the exact test by its short form where that is clear of a tie: outside a margin of four times
+    // the two forms' errors (the float form's follows the size of its uncombined terms, about |k - m|
+    // each), which leaves about one test in 1000 to the float form itself
+    const float n2 = n + 2.f;
+    const float np2 = n2 * p;
+    const float d = (np2 - (k + 1.f)) + fmaf(n2, p, -np2);
+    float size;
+    const float ex = btrs_excess(n, k, m, q, d, v1, us, aa, bb, spq, size);
+    const bool accept = fabsf(ex) > fmaf(size + 3.f * fabsf(k - m), 0x1p-19f, 0x1p-16f)
+                            ? ex > 0.f
+                            : btrs_exact_f32(n, p, k, us, v1, aa, bb, spq);
+    if (accept) return k;
   }
 }
 
