@@ -296,25 +296,6 @@ struct BinomWordsF {
   }
 };
 
-// BTRS's exact test in float (true: accept)
-static __device__ __noinline__ bool btrs_exact_f32(float n, float p, float k, float us, float v1, float aa, float bb,
-                                                   float spq) {
-  const float q = 1.f - p;
-  const float m = floorf(fmaf(n, p, p));  // floor((n + 1) p), one rounding
-  const float fcm = stirling_fc(m) + stirling_fc(n - m);
-  const float alpha = (2.83f + __fdividef(5.1f, bb)) * spq;
-  const float n2 = n + 2.f;
-  const float np2 = n2 * p;
-  const float np2_err = fmaf(n2, p, -np2);  // (n + 2) p = np2 + np2_err exactly
-  const float d = ((np2 - (k + 1.f)) + np2_err);
-  const float lr = (m + 0.5f) * log1pf(__fdividef(m - k, k + 1.f)) +
-                   (n - m + 0.5f) * log1pf(__fdividef(k - m, n - k + 1.f)) +
-                   (k - m) * log1pf(__fdividef(d, (k + 1.f) * q)) + fcm - stirling_fc(k) -
-                   stirling_fc(n - k);
-  const float v = logf(__fdividef(v1 * alpha, __fdividef(aa, us * us) + bb));
-  return v <= lr;
-}
-
 static __device__ __noinline__ float binomial_half_f32(float n, float p, BinomWordsF& b) {
   const float q = 1.f - p;
   if (n * p < 10.f) {
@@ -340,7 +321,9 @@ static __device__ __noinline__ float binomial_half_f32(float n, float p, BinomWo
   const float c = n * p + 0.5f;
   const float ci = floorf(c), cf = c - ci;
   const float vr = 0.92f - __fdividef(4.2f, bb);
-  const float m = floorf(fmaf(n, p, p));  // floor((n + 1) p), one rounding
+  const float mode = floorf(fmaf(n, p, p));
+  bool have_m = false;
+  float m = 0.f, fcm = 0.f, alpha = 0.f, np2 = 0.f, np2_err = 0.f;
   for (;;) {
     const float u1 = b.next();
     const float v1 = b.next();
@@ -352,15 +335,29 @@ static __device__ __noinline__ float binomial_half_f32(float n, float p, BinomWo
     if (us >= 0.07f && v1 <= vr) return k;
     // the exact test by its short form where that is clear of a tie: outside a margin of four times
     // the two forms' errors (the float form's follows the size of its uncombined terms, about |k - m|
-    // each), which leaves about one test in 1000 to the float form itself
-    const float n2 = n + 2.f;
-    const float np2 = n2 * p;
-    const float d = (np2 - (k + 1.f)) + fmaf(n2, p, -np2);
+    // each), which leaves about one test in 1000 to the float form
+    const float e2 = __fmul_rn(n + 2.f, p);
     float size;
-    const float ex = btrs_excess(n, k, m, q, d, v1, us, aa, bb, spq, size);
-    const bool accept = fabsf(ex) > fmaf(size + 3.f * fabsf(k - m), 0x1p-19f, 0x1p-16f)
-                            ? ex > 0.f
-                            : btrs_exact_f32(n, p, k, us, v1, aa, bb, spq);
+    const float ex = btrs_excess(n, k, mode, q, __fsub_rn(e2, k + 1.f) + fmaf(n + 2.f, p, -e2), v1, us, aa, bb, spq, size);
+    bool accept = ex > 0.f;
+    if (!(fabsf(ex) > fmaf(size + 3.f * fabsf(k - mode), 0x1p-19f, 0x1p-16f))) {
+      if (!have_m) {
+        m = floorf(fmaf(n, p, p));  // floor((n + 1) p), one rounding
+        fcm = stirling_fc(m) + stirling_fc(n - m);
+        alpha = (2.83f + __fdividef(5.1f, bb)) * spq;
+        const float n2 = n + 2.f;
+        np2 = n2 * p;
+        np2_err = fmaf(n2, p, -np2);  // (n + 2) p = np2 + np2_err exactly
+        have_m = true;
+      }
+      const float d = ((np2 - (k + 1.f)) + np2_err);
+      const float lr = (m + 0.5f) * log1pf(__fdividef(m - k, k + 1.f)) +
+                       (n - m + 0.5f) * log1pf(__fdividef(k - m, n - k + 1.f)) +
+                       (k - m) * log1pf(__fdividef(d, (k + 1.f) * q)) + fcm - stirling_fc(k) -
+                       stirling_fc(n - k);
+      const float v = logf(__fdividef(v1 * alpha, __fdividef(aa, us * us) + bb));
+      accept = v <= lr;
+    }
     if (accept) return k;
   }
 }

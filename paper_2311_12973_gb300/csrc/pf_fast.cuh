@@ -35,16 +35,6 @@
 
 namespace smc2 {
 
-// floor(v) for a float 0 <= v <= 2^52 as its two 32-bit halves: hi = floor(v 2^-32)
-// and lo = floor(v - hi 2^32).  Both steps are exact in float (v 2^-32 is a power-of-
-// two scaling; v - hi 2^32 = v mod 2^32 holds at most v's 24 significant bits), and
-// the two 32-bit conversions avoid the float-to-u64 one, which runs on the FP64 pipe.
-__device__ __forceinline__ uint64_t floor_to_u64(float v) {
-  const float hi = floorf(v * 0x1p-32f);
-  const float lo = fmaf(-hi, 0x1p32f, v);
-  return ((uint64_t)__float2uint_rz(hi) << 32) | (uint64_t)__float2uint_rz(lo);
-}
-
 // 2^x by the hardware approximation (relative error about 2^-22; 0 for -inf).
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;

@@ -170,8 +170,15 @@ __device__ __forceinline__ double neg_inf<double>() {
   return -HUGE_VAL;
 }
 
-__device__ __forceinline__ uint64_t to_u64_rz(float v) { return __float2ull_rz(v); }
-__device__ __forceinline__ uint64_t to_u64_rz(double v) { return __double2ull_rz(v); }
+// floor(v) for a float 0 <= v <= 2^52 as its two 32-bit halves: hi = floor(v 2^-32)
+// and lo = floor(v - hi 2^32).  Both steps are exact in float (v 2^-32 is a power-of-
+// two scaling; v - hi 2^32 = v mod 2^32 holds at most v's 24 significant bits), and
+// the two 32-bit conversions avoid the float-to-u64 one, which runs on the FP64 pipe.
+__device__ __forceinline__ uint64_t floor_to_u64(float v) {
+  const float hi = floorf(v * 0x1p-32f);
+  const float lo = fmaf(-hi, 0x1p32f, v);
+  return ((uint64_t)__float2uint_rz(hi) << 32) | (uint64_t)__float2uint_rz(lo);
+}
 
 // u64 to float from its two 32-bit halves (relative error below 2^-23).
 __device__ __forceinline__ float u64_to_float(uint64_t v) {
@@ -650,6 +657,45 @@ __device__ __forceinline__ uint64_t quantise64(double a, int B, const Soft64Tabl
   return hi == 0u || (hi - 0x80000000u) < 0x40428000u ? m >> min(61 - B - min(k, 0), 63) : 0ull;
 }
 
+// A warp's sum of squared weights for the ESS test, c the thread's inclusive prefixes.  The test needs
+// the exact 128-bit sum (40 shuffles and adds) only near a tie; a sum of floats, within 2^-20 of it
+// (each weight reaches float to 2^-22, the squares and the sums over PPT, 5 and at most 16 terms
+// add a rounding each), decides the others.
+template <int PPT>
+__device__ __forceinline__ void store_q2_float(const uint64_t (&c)[PPT], int lane, float* out) {
+  float q2 = 0.f;
+  uint64_t prev = 0;
+#pragma unroll
+  for (int r = 0; r < PPT; ++r) {
+    const float q = u64_to_float(c[r] - prev);
+    prev = c[r];
+    q2 = fmaf(q, q, q2);
+  }
+  q2 = warp_sum(q2);
+  if (lane == 0) *out = q2;
+}
+__device__ __forceinline__ float total_q2_float(const unsigned __int128* wq2, int nw, int lane) {
+  return warp_sum(lane < nw ? *reinterpret_cast<const float*>(wq2 + lane) : 0.f);
+}
+template <int PPT>
+__device__ __forceinline__ void store_q2(const uint64_t (&c)[PPT], int lane, unsigned __int128* out) {
+  unsigned __int128 q2 = 0;
+  uint64_t prev = 0;
+#pragma unroll
+  for (int r = 0; r < PPT; ++r) {
+    const uint64_t q = c[r] - prev;
+    prev = c[r];
+    q2 += (unsigned __int128)q * q;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t lo = __shfl_xor_sync(0xffffffffu, (uint64_t)q2, o);
+    const uint64_t hi = __shfl_xor_sync(0xffffffffu, (uint64_t)(q2 >> 64), o);
+    q2 += ((unsigned __int128)hi << 64) | lo;
+  }
+  if (lane == 0) *out = q2;
+}
+
 // NAMED: groups wider than a warp that share a CTA synchronise on named
 // barriers 1..15 (ptxas then reserves all 16 barriers of the CTA, which limits
 // residency to four CTAs per SM).  Otherwise a wide group is the whole CTA and
@@ -818,7 +864,7 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
         if constexpr (F64)
           run += quantise64(l - m, B, tab);
         else
-          run += (l > neg_inf<R>()) ? to_u64_rz(fast_exp(l - m) * scaleB) : 0ull;
+          run += (l > neg_inf<R>()) ? floor_to_u64(fast_exp(l - m) * scaleB) : 0ull;
         P[lt * PPT + r] = run;
         StateVec<R, NS>::store(X, lt * PPT + r, x[r]);
       }
@@ -830,7 +876,7 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
 #pragma unroll
       for (int r = 0; r < PPT; ++r) {
         const R v = (ell[r] > neg_inf<R>()) ? fast_exp(ell[r] - m) * scaleB : (R)0;
-        run += to_u64_rz(v);
+        run += floor_to_u64(v);
         runf += (float)v;
         cf[r] = runf;
         c[r] = run;
@@ -843,24 +889,8 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
       for (int r = 0; r < PPT; ++r) P[lt * PPT + r] += excl;
     }
     if (lane == 31) wsum[warp] = incl;
-    if (adaptive) {  // the warp's sum of q^2, exact in 128 bits
-      unsigned __int128 q2 = 0;
-      if constexpr (!STAGED) {
-        uint64_t prev = 0;
-#pragma unroll
-        for (int r = 0; r < PPT; ++r) {
-          const uint64_t qv = c[r] - prev;
-          prev = c[r];
-          q2 += (unsigned __int128)qv * qv;
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const uint64_t lo = __shfl_xor_sync(0xffffffffu, (uint64_t)q2, o);
-        const uint64_t hi = __shfl_xor_sync(0xffffffffu, (uint64_t)(q2 >> 64), o);
-        q2 += ((unsigned __int128)hi << 64) | lo;
-      }
-      if (lane == 0) wq2[warp] = q2;
+    if constexpr (GEN) {
+      if (adaptive) store_q2_float<PPT>(c, lane, reinterpret_cast<float*>(wq2 + warp));
     }
     group_sync();
     // total S, and the weight `base` of the warps before this one: an inclusive
@@ -893,17 +923,21 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
     // the schedule: every step, or when the ESS of the integer weights (Eq. 12) is below
     // pf_ess_frac M (by lane 0 of every warp, from the same totals, so the whole group decides alike)
     bool resample = t < T;
-    if (adaptive && resample) {
-      int below = 0;
-      if (lane == 0) {
-        unsigned __int128 Q2 = 0;
-        for (int w = 0; w < nw; ++w) Q2 += wq2[w];
-        // the test of Eq. (12) in float: S^2 < threshold sum q^2
-        const float q2 = fmaf(__ull2float_rn((uint64_t)(Q2 >> 64)), 0x1p64f, __ull2float_rn((uint64_t)Q2));
-        const float Sf = u64_to_float(S);
-        below = Sf * Sf < ess_thr * q2;
+    if constexpr (GEN) {
+      if (adaptive && resample) {
+        // the test of Eq. (12) as S^2 < threshold sum q^2, from sums in float; near a tie from the exact sum
+        const float Sf = u64_to_float(S), rhs = ess_thr * total_q2_float(wq2, nw, lane);
+        resample = Sf * Sf < rhs;
+        if (!(fabsf(Sf * Sf - rhs) > 0x1p-16f * rhs)) {
+          group_sync();  // the float sums are read
+          store_q2<PPT>(c, lane, wq2 + warp);
+          group_sync();
+          unsigned __int128 Q2 = 0;
+          for (int w = 0; w < nw; ++w) Q2 += wq2[w];
+          const float q2 = fmaf(__ull2float_rn((uint64_t)(Q2 >> 64)), 0x1p64f, __ull2float_rn((uint64_t)Q2));
+          resample = Sf * Sf < ess_thr * q2;
+        }
       }
-      resample = __shfl_sync(0xffffffffu, below, 0) != 0;
     }
     if constexpr (GEN) {
       if (resample) Lc = loglik;  // Eq. (13): every particle will carry the mean weight (thread 0)
@@ -1262,23 +1296,7 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
     const uint64_t incl = warp_incl_scan_u64(run, lane);
     const uint64_t excl = incl - run;
     if (lane == 31) wsum[warp] = incl;
-    if (adaptive) {  // the warp's sum of q^2, exact in 128 bits
-      unsigned __int128 q2 = 0;
-      uint64_t prev = 0;
-#pragma unroll
-      for (int r = 0; r < PPT; ++r) {
-        const uint64_t qv = c[r] - prev;
-        prev = c[r];
-        q2 += (unsigned __int128)qv * qv;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const uint64_t lo = __shfl_xor_sync(0xffffffffu, (uint64_t)q2, o);
-        const uint64_t hi = __shfl_xor_sync(0xffffffffu, (uint64_t)(q2 >> 64), o);
-        q2 += ((unsigned __int128)hi << 64) | lo;
-      }
-      if (lane == 0) wq2[warp] = q2;
-    }
+    if (adaptive) store_q2_float<PPT>(c, lane, reinterpret_cast<float*>(wq2 + warp));
     group_sync();
     // total S, and the weight `base` of the warps before this one
     uint64_t wpre = lane < nw ? wsum[lane] : 0ull;
@@ -1294,25 +1312,22 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
     inc_m = mine ? m : inc_m;
     inc_S = mine ? S : inc_S;
     // the schedule: every step, or when the ESS of the integer weights (Eq. 12) is below
-    // pf_ess_frac M, formed with the same correctly rounded operations as the oracle (by
-    // lane 0 of every warp, from the same totals, so the whole group decides alike)
+    // pf_ess_frac M: from sums in float, and near a tie from the exact sum of q^2 with the same
+    // correctly rounded operations as the oracle (the whole group sees the same totals)
     bool resample = t < TT;
     if (adaptive && resample) {
-      int below = 0;
-      if (lane == 0) {
+      const float Sf = u64_to_float(S), rhs = ess_thr * total_q2_float(wq2, nw, lane);
+      resample = Sf * Sf < rhs;
+      if (!(fabsf(Sf * Sf - rhs) > 0x1p-16f * rhs)) {
+        group_sync();  // the float sums are read
+        store_q2<PPT>(c, lane, wq2 + warp);
+        group_sync();
         unsigned __int128 Q2 = 0;
         for (int w = 0; w < nw; ++w) Q2 += wq2[w];
-        // in float first, whose error here is below 2^-20: only a near tie needs FP64
-        const float q2f = fmaf(u64_to_float((uint64_t)(Q2 >> 64)), 0x1p64f, u64_to_float((uint64_t)Q2));
-        const float Sf = u64_to_float(S), lhs = Sf * Sf, rhs = ess_thr * q2f;
-        below = lhs < rhs;
-        if (!(fabsf(lhs - rhs) > 0x1p-18f * rhs)) {
-          const double q2 = (double)(uint64_t)(Q2 >> 64) * 0x1p64 + (double)(uint64_t)Q2;
-          const double ess = __ddiv_rn((double)S * (double)S, q2);
-          below = ess < mdl.pf_ess_frac * (double)M;
-        }
+        const double q2 = (double)(uint64_t)(Q2 >> 64) * 0x1p64 + (double)(uint64_t)Q2;
+        const double ess = __ddiv_rn((double)S * (double)S, q2);
+        resample = ess < mdl.pf_ess_frac * (double)M;
       }
-      resample = __shfl_sync(0xffffffffu, below, 0) != 0;
     }
     inc_res = mine ? resample : inc_res;
     from = resample ? (multinomial ? 2 : 1) : 0;
