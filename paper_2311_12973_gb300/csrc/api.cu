@@ -429,8 +429,7 @@ smc2_status choose_launch_shape(smc2_ctx* c) {
     PFLaunch L = c->pl;
     L.t_cap = t_cap;
     float ms = 0.f;
-    const bool ok = cudaMemsetAsync(c->d_wu_counter, 0, sizeof(int), s) == cudaSuccess &&
-                    cudaEventRecord(e0, s) == cudaSuccess && ctx_pf_launch(c, c->pf_grid, L, s) == cudaSuccess &&
+    const bool ok = cudaEventRecord(e0, s) == cudaSuccess && ctx_pf_launch(c, c->pf_grid, L, s) == cudaSuccess &&
                     cudaEventRecord(e1, s) == cudaSuccess && cudaEventSynchronize(e1) == cudaSuccess &&
                     cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
     c->kernel_launches++;
@@ -497,6 +496,7 @@ smc2_status clear_run_state(smc2_ctx* c) {
   SMC2_TRY(cudaMemsetAsync(c->d_k, 0, 4 * sizeof(int), s));
   SMC2_TRY(cudaMemsetAsync(c->d_status, 0, 4 * sizeof(int), s));
   SMC2_TRY(cudaMemsetAsync(c->d_grid_ticket, 0, 4 * sizeof(unsigned), s));
+  SMC2_TRY(cudaMemsetAsync(c->d_wu_counter, 0, 4 * sizeof(int), s));
   for (int d = 0; d < c->n_ds; ++d) {
     const DSDev& ds = c->h_ds[d];
     SMC2_TRY(cudaMemsetAsync(ds.tickets, 0, 4 * sizeof(unsigned), s));
@@ -596,7 +596,6 @@ smc2_status enqueue_iteration(smc2_ctx* c, cudaStream_t s, cudaEvent_t ev0, cuda
   SMC2_TRY(cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0));
   SMC2_TRY(outer_lkfit(c->op, c->side_stream));
   SMC2_TRY(cudaEventRecord(c->ev_join, c->side_stream));
-  SMC2_TRY(cudaMemsetAsync(c->d_wu_counter, 0, sizeof(int), s));
   if (ev0) SMC2_TRY(cudaEventRecordWithFlags(ev0, s, cudaEventRecordExternal));
   SMC2_TRY(ctx_pf_launch(c, c->pf_grid, c->pl, s));
   if (ev1) SMC2_TRY(cudaEventRecordWithFlags(ev1, s, cudaEventRecordExternal));
@@ -846,6 +845,8 @@ static smc2_status pf_standalone(smc2_ctx* c, const double* theta, int n, int it
   }
   const int occ = std::max(1, ctx_pf_occupancy(c, trace));
   const int grid = std::min(L.n_wu, occ * c->sms);
+  // more units than fit at once: from the queue, so that CTAs with light filters take more of them
+  if (L.n_wu > grid) L.wu_counter = c->d_wu_counter;
   SMC2_TRY(ctx_pf_launch(c, grid, L, c->stream, trace));
   c->kernel_launches++;
   return SMC2_OK;

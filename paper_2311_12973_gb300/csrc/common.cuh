@@ -171,6 +171,18 @@ __device__ __forceinline__ void named_barrier(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// Called by every CTA of a dynamically scheduled launch when the queue is empty: the last one
+// leaves the queue's two counters at zero for the next launch, which saves a memset per launch.
+__device__ __forceinline__ void release_queue(int* counter) {
+  if (counter && threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(counter + 1, 1) == (int)gridDim.x - 1) {
+      counter[0] = 0;
+      counter[1] = 0;
+    }
+  }
+}
+
 __device__ __forceinline__ void raise_status(int* status, int bits) {
   if (status) atomicOr(status, bits);
 }

@@ -144,7 +144,8 @@ struct PFLaunch {
   const int4* wus;     // (job, first filter, count, -); NULL: one job, unit w = filters [w*fpc, ...)
   int n_wu;
   int fpc_single;      // filters per unit when wus == NULL
-  int* wu_counter;     // dynamic scheduling when not NULL
+  int* wu_counter;     // dynamic scheduling when not NULL: [0] next unit, [1] CTAs finished; both 0
+                       // before a launch, and again after it (the last CTA clears them)
   uint64_t seed;
   const int* k_done;   // iteration = *k_done + 1 when not NULL
   int k_imm;

@@ -111,7 +111,7 @@ extern "C" smc2_status smc2_pf_loglik_noalloc(const smc2_config* cfg, const doub
     return fail(SMC2_ECUDA, "device query");
 
   // the previous call's counter is still in the array: start it from zero
-  e = cudaMemsetAsync(counter, 0, sizeof(int), s);
+  e = cudaMemsetAsync(counter, 0, 2 * sizeof(int), s);
   if (e != cudaSuccess) return fail(SMC2_ECUDA, cudaGetErrorString(e));
   e = outer_obs_terms(cfg->precision, model, y_dev, cfg->T, obs, s);
   if (e != cudaSuccess) return fail(SMC2_ECUDA, cudaGetErrorString(e));

@@ -572,6 +572,7 @@ __global__ void __maxnreg__((FastRegCap<PPT, GROUPED>::value)) pf_fast_kernel(PF
     }
     if (!L.wu_counter) __syncthreads();
   }
+  release_queue(L.wu_counter);
 }
 
 template <int MODEL, bool TRACE, bool GROUPED>

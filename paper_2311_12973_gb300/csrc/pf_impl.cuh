@@ -1457,6 +1457,7 @@ __global__ void __maxnreg__((RegCap<R, PPT>::value)) pf_kernel(PFLaunch L) {
     }
     if (!L.wu_counter) __syncthreads();
   }
+  release_queue(L.wu_counter);
 }
 
 
