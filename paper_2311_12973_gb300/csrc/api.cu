@@ -37,6 +37,11 @@ constexpr double kMlpLr = 5e-3;
 constexpr int kMlpSteps = 16;
 constexpr int kMlpWindow = 4;
 
+// Read-backs go through one page-locked buffer of the context where they fit: copies into it are
+// queued without waiting, so a call of several costs one wait (a copy into pageable memory waits
+// by itself: 16 us each, 20 of them after a run of 20 iterations).
+constexpr size_t kPinnedBytes = 256 * 1024;
+
 struct GraphKey {
   int n_iter, timing;
   bool operator<(const GraphKey& o) const {
@@ -76,6 +81,7 @@ struct smc2_ctx {
   int* d_wu_counter = nullptr;
   int* d_k = nullptr;
   int* d_status = nullptr;
+  char* pinned = nullptr;   // page-locked staging of read-backs (kPinnedBytes)
   unsigned* d_grid_ticket = nullptr;
   int ppt = 4, pf_block = 256, pf_grid = 1;
   bool pf_named = false;    // pf_kernel: named-barrier groups; the FP32 filter: grouped instantiation
@@ -663,12 +669,37 @@ void drop_graphs(smc2_ctx* c) {
   c->graphs.clear();
 }
 
-smc2_status sticky(smc2_ctx* c) {
-  int bits = 0;
-  SMC2_TRY(cudaMemcpyAsync(&bits, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  SMC2_TRY(cudaStreamSynchronize(c->stream));
-  return status_from_bits(bits);
-}
+// The pieces of one read-back: device ranges copied to host places, then one wait and the sticky
+// device status.
+struct ReadBack {
+  smc2_ctx* c;
+  struct Piece {
+    void* dst;
+    const char* staged;
+    size_t bytes;
+  };
+  std::vector<Piece> pieces;
+  size_t used = sizeof(double);  // the status word leads the buffer
+  explicit ReadBack(smc2_ctx* ctx) : c(ctx) {}
+  cudaError_t add(void* dst, const void* src, size_t bytes) {
+    if (!dst || !bytes) return cudaSuccess;
+    if (used + bytes > kPinnedBytes) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, c->stream);
+    char* at = c->pinned + used;
+    used += (bytes + 15) & ~(size_t)15;
+    pieces.push_back({dst, at, bytes});
+    return cudaMemcpyAsync(at, src, bytes, cudaMemcpyDeviceToHost, c->stream);
+  }
+  smc2_status finish() {
+    SMC2_TRY(cudaMemcpyAsync(c->pinned, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    SMC2_TRY(cudaStreamSynchronize(c->stream));
+    for (const Piece& p : pieces) memcpy(p.dst, p.staged, p.bytes);
+    int bits = 0;
+    memcpy(&bits, c->pinned, sizeof(int));
+    return status_from_bits(bits);
+  }
+};
+
+smc2_status sticky(smc2_ctx* c) { return ReadBack(c).finish(); }
 
 bool bad_ds(const smc2_ctx* c, int d) { return !c || d < 0 || d >= c->n_ds; }
 
@@ -741,6 +772,7 @@ smc2_status smc2_init(const smc2_config* cfg, const double* y, void* stream, smc
       cudaEventCreateWithFlags(&c->ev_tjoin, cudaEventDisableTiming) != cudaSuccess)
     return fail(SMC2_ECUDA);
 
+  if (cudaMallocHost(&c->pinned, kPinnedBytes) != cudaSuccess) return fail(SMC2_ENOMEM);
   c->arena_bytes = layout(c, nullptr);
   if (cudaMalloc(&c->arena, c->arena_bytes) != cudaSuccess) return fail(SMC2_ENOMEM);
   layout(c, c->arena);
@@ -890,11 +922,18 @@ smc2_status smc2_run(smc2_ctx* c, int n_iter, smc2_iter_stats* stats_host) {
     }
   }
   if (stats_host) {
+    ReadBack rb(c);
+    if (c->n_ds == 1) {
+      SMC2_TRY(rb.add(stats_host, c->h_ds[0].hist + k0, (size_t)n_iter * sizeof(smc2_iter_stats)));
+      return rb.finish();
+    }
+    std::vector<smc2_iter_stats> h((size_t)c->n_ds * n_iter);  // dataset-major, as on the device
     for (int d = 0; d < c->n_ds; ++d)
-      for (int i = 0; i < n_iter; ++i)
-        SMC2_TRY(cudaMemcpyAsync(stats_host + (size_t)i * c->n_ds + d, c->h_ds[d].hist + k0 + i,
-                                 sizeof(smc2_iter_stats), cudaMemcpyDeviceToHost, c->stream));
-    return sticky(c);
+      SMC2_TRY(rb.add(h.data() + (size_t)d * n_iter, c->h_ds[d].hist + k0, (size_t)n_iter * sizeof(smc2_iter_stats)));
+    const smc2_status done = rb.finish();
+    for (int d = 0; d < c->n_ds; ++d)
+      for (int i = 0; i < n_iter; ++i) stats_host[(size_t)i * c->n_ds + d] = h[(size_t)d * n_iter + i];
+    return done;
   }
   return SMC2_OK;
 }
@@ -911,9 +950,10 @@ smc2_status smc2_estimate(smc2_ctx* c, int dataset, double* mean_host, double* l
   const int D = c->D;
   smc2_iter_stats last;
   std::vector<double> rec((size_t)1 + D + D * D);
-  SMC2_TRY(cudaMemcpyAsync(&last, s.hist + (c->k_host - 1), sizeof(last), cudaMemcpyDeviceToHost, c->stream));
-  SMC2_TRY(cudaMemcpyAsync(rec.data(), s.rec, rec.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  const smc2_status st = sticky(c);
+  ReadBack rb(c);
+  SMC2_TRY(rb.add(&last, s.hist + (c->k_host - 1), sizeof(last)));
+  SMC2_TRY(rb.add(rec.data(), s.rec, rec.size() * sizeof(double)));
+  const smc2_status st = rb.finish();
   const double l = rec[0];
   // recycled mean and covariance: the l_k-weighted first and second moments (Eq. 29)
   for (int d = 0; d < D; ++d) {
@@ -943,11 +983,12 @@ smc2_status smc2_get_state(smc2_ctx* c, int dataset, int* k_out, double* theta, 
   const DSDev& s = c->h_ds[dataset];
   const int N = s.N, D = c->D;
   std::vector<double> soa((size_t)D * N);
-  SMC2_TRY(cudaMemcpyAsync(soa.data(), s.thA, soa.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  if (lp) SMC2_TRY(cudaMemcpyAsync(lp, s.lpA, N * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  if (ll) SMC2_TRY(cudaMemcpyAsync(ll, s.llA, N * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  if (lw) SMC2_TRY(cudaMemcpyAsync(lw, s.logw, N * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-  smc2_status st = sticky(c);
+  ReadBack rb(c);
+  SMC2_TRY(rb.add(soa.data(), s.thA, soa.size() * sizeof(double)));
+  SMC2_TRY(rb.add(lp, s.lpA, N * sizeof(double)));
+  SMC2_TRY(rb.add(ll, s.llA, N * sizeof(double)));
+  SMC2_TRY(rb.add(lw, s.logw, N * sizeof(double)));
+  smc2_status st = rb.finish();
   if (theta)
     for (int i = 0; i < N; ++i)
       for (int d = 0; d < D; ++d) theta[(size_t)i * D + d] = soa[(size_t)d * N + i];
@@ -1184,6 +1225,7 @@ void smc2_destroy(smc2_ctx* c) {
   if (c->stream || c->arena) cudaStreamSynchronize(c->stream);
   drop_graphs(c);
   if (c->arena) cudaFree(c->arena);
+  if (c->pinned) cudaFreeHost(c->pinned);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);

@@ -51,9 +51,9 @@ class IterStats(C.Structure):
     def as_dict(self, D: int) -> dict:
         return {"k": self.k, "resampled": self.resampled, "lk_fallback": self.lk_fallback,
                 "dataset": self.dataset, "ess": self.ess, "lse": self.lse, "lse2": self.lse2,
-                "logz": self.logz, "est": np.array(self.est[:D]), "mlp_used": self.mlp_used,
+                "logz": self.logz, "est": np.frombuffer(self.est)[:D].copy(), "mlp_used": self.mlp_used,
                 "mlp_loss": self.mlp_loss,
-                "cov": np.array(self.cov[:]).reshape(MAX_D, MAX_D)[:D, :D].copy()}
+                "cov": np.frombuffer(self.cov).reshape(MAX_D, MAX_D)[:D, :D].copy()}
 
 
 class SMC2Error(RuntimeError):
