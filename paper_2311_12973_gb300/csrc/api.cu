@@ -577,6 +577,7 @@ void fill_params(smc2_ctx* c) {
   L.mdl.i0 = c->cfg.i0;
   L.mdl.lambda_floor = c->cfg.lambda_floor;
   L.mdl.n_sub = c->cfg.n_sub;
+  pf_model_constants(L.mdl);
   L.mdl.pf_scheme = c->cfg.pf_scheme;
   L.mdl.pf_ess_frac = c->cfg.pf_ess_frac;
 }

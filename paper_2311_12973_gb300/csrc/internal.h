@@ -134,10 +134,19 @@ constexpr int kTraceState = 5;  // floats per particle in a state trace
 
 struct PFModel {
   double npop, e0, i0, lambda_floor;
+  double inv_npop, dt;        // 1 / npop, 1 / n_sub (pf_model_constants)
+  float inv_npop_f32, dt_f32; // the same rounded to float
   int n_sub;
   int pf_scheme;       // PF resampling: 0 systematic, 1 multinomial
   double pf_ess_frac;  // <= 0: every step; else when the ESS is below pf_ess_frac * M
 };
+
+inline void pf_model_constants(PFModel& m) {
+  m.inv_npop = 1.0 / m.npop;
+  m.dt = 1.0 / m.n_sub;
+  m.inv_npop_f32 = (float)m.inv_npop;
+  m.dt_f32 = (float)m.dt;
+}
 
 struct PFLaunch {
   const PFJob* jobs;   // NULL: the single job job0

@@ -140,6 +140,7 @@ extern "C" smc2_status smc2_pf_loglik_noalloc(const smc2_config* cfg, const doub
   L.mdl.i0 = cfg->i0;
   L.mdl.lambda_floor = cfg->lambda_floor;
   L.mdl.n_sub = cfg->n_sub;
+  pf_model_constants(L.mdl);
   L.mdl.pf_scheme = cfg->pf_scheme;
   L.mdl.pf_ess_frac = cfg->pf_ess_frac;
   L.t_cap = 0;

@@ -97,7 +97,7 @@ template <typename R, int PPT>
 struct RegCap {
   static constexpr int value =
       sizeof(R) == 4 ? (PPT <= 2 ? 64 : (PPT == 4 ? 96 : (PPT == 8 ? 128 : 168)))
-                     : (PPT <= 4 ? 80 : (PPT == 8 ? 128 : 168));
+                     : (PPT == 1 ? 128 : PPT <= 4 ? 80 : (PPT == 8 ? 128 : 168));
   static_assert(PPT == 1 || PPT == 2 || PPT == 4 || PPT == 8 || PPT == 16, "particles per thread");
 };
 
@@ -251,14 +251,28 @@ __device__ __forceinline__ double fast_exp(double x) { return exp(x); }
 template <typename R, int MODEL>
 struct FilterParams;
 
+// e^a[0] .. e^a[N - 1], the same in every lane: one evaluation, lane k's argument a[k] (every warp of
+// a filter forms them, and an exponential is about 17 FP64 instructions of 19 clocks each).
+template <int N>
+__device__ __forceinline__ void warp_exps(const double* a, double* out) {
+  const int lane = threadIdx.x & 31;
+  double v = a[0];
+#pragma unroll
+  for (int n = 1; n < N; ++n) v = lane == n ? a[n] : v;
+  v = exp(v);
+#pragma unroll
+  for (int n = 0; n < N; ++n) out[n] = __shfl_sync(0xffffffffu, v, n);
+}
+
 template <typename R>
 struct FilterParams<R, MODEL_LG> {
   R phi, sx, inv_sy, c_obs;
   __device__ void load(const double* th, const PFModel&) {
-    const double sy = exp(th[2]);
+    double e[2];  // sigma_x, sigma_y
+    warp_exps<2>(th + 1, e);
     phi = (R)th[0];
-    sx = (R)exp(th[1]);
-    inv_sy = (R)(1.0 / sy);
+    sx = (R)e[0];
+    inv_sy = (R)(1.0 / e[1]);
     c_obs = (R)(-0.5 * kLog2Pi - th[2]);
   }
   __device__ __forceinline__ void init(R* x, R z0, const double*) const { x[0] = z0; }
@@ -275,12 +289,14 @@ struct FilterParams<R, MODEL_SEIR> {
   R srw, kappa, gamma, inv_npop, dt, lam_floor, S0, E0, I0, lb0;
   int n_sub;
   __device__ void load(const double* th, const PFModel& m) {
+    double e[3];
+    warp_exps<3>(th + 1, e);
     lb0 = (R)th[0];
-    srw = (R)exp(th[1]);
-    kappa = (R)exp(th[2]);
-    gamma = (R)exp(th[3]);
-    inv_npop = (R)(1.0 / m.npop);
-    dt = (R)(1.0 / m.n_sub);
+    srw = (R)e[0];
+    kappa = (R)e[1];
+    gamma = (R)e[2];
+    inv_npop = m.inv_npop_f32;
+    dt = m.dt_f32;
     n_sub = m.n_sub;
     lam_floor = (R)m.lambda_floor;
     S0 = (R)(m.npop - m.e0 - m.i0);
@@ -340,7 +356,7 @@ struct SeirDay {
 static __device__ __noinline__ SeirDay seir_day_fp64(SeirDay s, double log_beta, double th2, double th3,
                                                      const PFModel& m) {
   const double beta = exp(log_beta), kappa = exp(th2), gamma = exp(th3);
-  const double inv_npop = 1.0 / m.npop, dt = 1.0 / m.n_sub;
+  const double inv_npop = m.inv_npop, dt = m.dt;
   s.lam = 0.0;
   for (int n = 0; n < m.n_sub; ++n) {
     const double infection = beta * s.S * s.I * inv_npop;
@@ -387,8 +403,10 @@ struct FilterParams<double, MODEL_SEIR> {
     lb0 = th[0];
     th2 = th[2];
     th3 = th[3];
-    srw = exp(th[1]);
-    const double dt = 1.0 / m.n_sub, kdt = exp(th[2]) * dt, gdt = exp(th[3]) * dt;
+    double e[3];
+    warp_exps<3>(th + 1, e);
+    srw = e[0];
+    const double dt = m.dt, kdt = e[1] * dt, gdt = e[2] * dt;
     nkdt = -kdt;
     ngdt = -gdt;
     n_sub = m.n_sub;
@@ -497,10 +515,11 @@ template <>
 struct FilterParams<double, MODEL_LG> {
   double phi, sx, inv_sy, c_obs;
   __device__ void load(const double* th, const PFModel&) {
-    const double sy = exp(th[2]);
+    double e[2];  // sigma_x, sigma_y
+    warp_exps<2>(th + 1, e);
     phi = th[0];
-    sx = exp(th[1]);
-    inv_sy = 1.0 / sy;
+    sx = e[0];
+    inv_sy = 1.0 / e[1];
     c_obs = -0.5 * kLog2Pi - th[2];
   }
   __device__ __forceinline__ void init(double* x, double z0, const double*) const { x[0] = z0; }
@@ -749,7 +768,7 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
   const int B = fixed_point_bits(M);
   const int log2M = ((M & (M - 1)) == 0) ? (__ffs(M) - 1) : -1;
   const R scaleB = (R)ldexp(1.0, B);
-  const double log_norm = -(double)B * kLn2 - log((double)M);
+  const double log_norm = warp == 0 ? -(double)B * kLn2 - log((double)M) : 0.0;  // thread 0's
   const R4* obs = reinterpret_cast<const R4*>(J.obs);
 
   R x[PPT][NS];
@@ -1154,7 +1173,6 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
   const uint32_t c3multi = counter_c3(TAG_PF_MULTI, k);
   const uint32_t c3binom = counter_c3(TAG_PF_BINOM, k);
   const int B = fixed_point_bits(M);
-  const double log_norm = -(double)B * kLn2 - log((double)M);
   const Double4* obs = reinterpret_cast<const Double4*>(J.obs);
 #pragma unroll 1
   for (int r = 0; r < PPT; ++r) {
@@ -1180,8 +1198,8 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
   bool dead = false;
   int from = 0;  // where the next step's states come from: 0 their own slot, 1 the marks, 2 mark[] as it stands
   // Likelihood increments: lane (t - 1) % 32 of the group's first warp keeps step t's maximum and
-  // total, and every 32 steps the lanes take their logarithms side by side and the sum runs over
-  // them in step order (a logarithm by one lane each step would cost that warp its full time).
+  // total, and every 32 steps the lanes take their logarithms side by side and are summed (a
+  // logarithm by one lane each step would cost that warp its full time).
   double inc_m = 0.0;
   uint64_t inc_S = 1;
   bool inc_res = false;
@@ -1191,22 +1209,29 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
     // max + log(S 2^-B) - log M, log S from its binary exponent and mantissa
     const int e = 63 - __clzll((long long)inc_S);
     const double mant = (double)(e >= 52 ? (inc_S >> (e - 52)) : (inc_S << (52 - e))) * 0x1p-52;
-    const double lmean = inc_m + ((double)e * kLn2 + log(mant)) + log_norm;
-    double delta = 0.0;
-    for (int s = 0; s < n; ++s) {
-      const double v = __shfl_sync(0xffffffffu, lmean, s);
-      if constexpr (GENERAL) {
-        const double logp_prev = loglik;
-        loglik = Lc + v;
-        if (lane == s) delta = loglik - logp_prev;
-        if (__shfl_sync(0xffffffffu, (int)inc_res, s)) Lc = loglik;  // Eq. (13): the mean weight from here on
-      } else {
-        loglik += v;
-        if (lane == s) delta = v;
+    const double lmean = lane < n ? inc_m + ((double)e * kLn2 + log(mant)) + (-(double)B * kLn2 - log((double)M)) : 0.0;
+    if constexpr (GENERAL) {
+      // Eq. (13): a resampling step's estimate is the common weight from there on, so the steps since
+      // the last one are replaced by the latest
+      const uint32_t res = __ballot_sync(0xffffffffu, inc_res && lane < n);
+      if (J.delta) {  // estimates after each step: the increments of the resampling steps before it
+        double before = Lc, prev = loglik;
+        for (int s = 0; s < n; ++s) {
+          const double v = before + __shfl_sync(0xffffffffu, lmean, s);
+          if (lane == 0) J.delta[(size_t)i * TT + t0 + s] = v - prev;
+          prev = v;
+          if (res & (1u << s)) before = v;
+        }
       }
+      const double last = __shfl_sync(0xffffffffu, lmean, n - 1);
+      Lc += warp_sum((res >> lane) & 1u ? lmean : 0.0);
+      loglik = (res >> (n - 1)) & 1u ? Lc : Lc + last;
+    } else {
+      if (J.delta && lane < n) J.delta[(size_t)i * TT + t0 + lane] = lmean;
+      loglik += warp_sum(lmean);
     }
-    if (J.delta && lane < n) J.delta[(size_t)i * TT + t0 + lane] = delta;
   };
+  Double4 ob_next = obs[0];
 
   for (int t = 1; t <= TT; ++t) {
     if (((t - 1) & 31) == 0) add_increments(t - 1);
@@ -1220,7 +1245,8 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
     uint32_t* sUg = sU + 4 * (((t - 1) >> 2) & 1);  // resampling words of four steps
     if (tm == 0 && lt < 4 && t + lt < TT)
       sUg[lt] = philox4x32_10(make_uint4(0u, (uint32_t)(t + lt), c2, c3res), key).x;
-    const Double4 ob = obs[t - 1];
+    const Double4 ob = PPT == 1 ? ob_next : obs[t - 1];
+    if (PPT == 1) ob_next = obs[min(t, TT - 1)];  // in flight during the step
     double lmax = neg_inf<double>();
     uint32_t a = carry[lt];
 #pragma unroll 1
@@ -1228,8 +1254,8 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
       const int j = lt * PPT + r, pos = r * T + lt;
       if (Rg::kZ && tm == 0) {  // one Philox call every four steps
         const uint4 w = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)((t - 1) >> 2), c2, c3prop), key);
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
+#pragma unroll (PPT == 1 ? 2 : 1)
+        for (int h = 0; h < 2; ++h) {  // the two pairs side by side where few warps are resident
           double z0, z1;
           s64_normal_pair(h ? w.z : w.x, h ? w.w : w.y, tab, z0, z1);
           Z[(size_t)(2 * h) * Mp + pos] = z0;
@@ -1401,11 +1427,11 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
 template <bool SHARED>
 __device__ __forceinline__ const Soft64Tables& soft64_tables() {
   if constexpr (SHARED) {
-    __shared__ Soft64Tables s;
-    static_assert(sizeof(Soft64Tables) % 8 == 0, "copied by 8-byte words");
-    const uint64_t* from = reinterpret_cast<const uint64_t*>(&g_soft64);
-    uint64_t* to = reinterpret_cast<uint64_t*>(&s);
-    for (int w = threadIdx.x; w < (int)(sizeof(Soft64Tables) / 8); w += blockDim.x) to[w] = from[w];
+    __shared__ __align__(16) Soft64Tables s;
+    static_assert(sizeof(Soft64Tables) % 16 == 0, "copied by 16-byte words");
+    const uint4* from = reinterpret_cast<const uint4*>(&g_soft64);
+    uint4* to = reinterpret_cast<uint4*>(&s);
+    for (int w = threadIdx.x; w < (int)(sizeof(Soft64Tables) / 16); w += blockDim.x) to[w] = from[w];
     __syncthreads();
     return s;
   } else {
