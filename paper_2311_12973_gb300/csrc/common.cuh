@@ -94,6 +94,40 @@ __device__ __forceinline__ double uniform23<double>(uint32_t w) {
   return __longlong_as_double((long long)bits) - (1.0 - 0x1p-24);
 }
 
+// Hardware approximations without the instructions that treat subnormal numbers (none reaches
+// them here; otherwise the intrinsics' values).
+constexpr float kLn2F = 0.693147182464599609375f;
+__device__ __forceinline__ float ex2_approx(float x) {  // 2^x (relative error about 2^-22; 0 for -inf)
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {  // 1/x (about 1 ulp)
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float lg2_approx(float x) {  // log2 x
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float sin_approx(float x) {
+  float y;
+  asm("sin.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float cos_approx(float x) {
+  float y;
+  asm("cos.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 template <typename R>
 __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, R& z0, R& z1);
 // FP32: hardware approximations (lg2, rsqrt, sin, cos; absolute error about
@@ -102,12 +136,11 @@ __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, R& z0, R& z
 template <>
 __device__ __forceinline__ void box_muller<float>(uint32_t wa, uint32_t wb, float& z0, float& z1) {
   const float ua = uniform23<float>(wa), ub = uniform23<float>(wb);
-  const float e = -2.0f * __logf(ua);
-  const float r = e * rsqrtf(e);
-  float s, c;
-  __sincosf(6.28318530717958647692f * (ub - 0.5f), &s, &c);
-  z0 = -r * c;
-  z1 = -r * s;
+  const float e = lg2_approx(ua) * (-2.0f * kLn2F);
+  const float r = e * rsqrt_approx(e);
+  const float a = 6.28318530717958647692f * (ub - 0.5f);
+  z0 = -r * cos_approx(a);
+  z1 = -r * sin_approx(a);
 }
 template <>
 __device__ __forceinline__ void box_muller<double>(uint32_t wa, uint32_t wb, double& z0, double& z1) {

@@ -27,6 +27,12 @@
 //      after a barrier the ancestor of slot s is the largest current tag at or
 //      before s within its thread's slots -- ancestors never decrease along the
 //      slots -- and the thread reads that particle's state.
+// The step is bound by instruction issue (about 60 % of the slots; the rest waits on fixed
+// latencies and the three barriers).  What an instruction count bought last, same results bit for
+// bit: approximations without subnormal handling, packed Box-Muller, one fmaxf for NaN and the
+// first crossing's exact test from 64-by-32-bit products (6 wide multiplies where the 128-bit
+// comparison took 14): N=8192/M=1024/T=200 9.71 -> 9.55 ms, N=1001/M=300/T=73 (4 particles per
+// thread) 242.8 -> 233.7 us.
 // Shared arrays indexed by a slot or a particle s keep it at row s % PPT, column
 // s / PPT, so that a warp reading one entry per thread touches consecutive words.
 #pragma once
@@ -34,24 +40,6 @@
 #include "pf_impl.cuh"
 
 namespace smc2 {
-
-// 2^x by the hardware approximation (relative error about 2^-22; 0 for -inf).
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-__device__ __forceinline__ float rcp_approx(float x) {  // 1/x, hardware approximation (about 1 ulp)
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float lg2_approx(float x) {  // log2 x, hardware approximation
-  float y;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 __device__ __forceinline__ float2 bc2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -104,7 +92,8 @@ struct PairModel<MODEL_SEIR> {
   __device__ __forceinline__ float2 step(float2* x, float2 z, const float4& ob, float2& lam, float2& d,
                                          int& far) const {
     x[3] = fma2(srw, z, x[3]);
-    const float2 beta = make_float2(__expf(x[3].x), __expf(x[3].y));
+    const float2 le = mul2(x[3], bc2(1.4426950408889634f));
+    const float2 beta = make_float2(ex2_approx(le.x), ex2_approx(le.y));
     float2 S = x[0], E = x[1], I = x[2];
     lam = bc2(0.f);
     if (n_sub == 2) {
@@ -162,6 +151,18 @@ __device__ __forceinline__ void normals4_rk(uint4 c, const uint32_t (&rk)[20], f
   const uint4 w = philox4x32_10_rk(c, rk);
   box_muller<float>(w.x, w.y, z[0], z[1]);
   box_muller<float>(w.z, w.w, z[2], z[3]);
+}
+// box_muller<float> of two particles' words, side by side in packed instructions
+__device__ __forceinline__ void box_muller2(uint32_t wa0, uint32_t wa1, uint32_t wb0, uint32_t wb1, float2& z0,
+                                            float2& z1) {
+  const float2 one = bc2(-(1.0f - 0x1p-24f));
+  const float2 ua = add2(make_float2(__uint_as_float(0x3f800000u | (wa0 >> 9)), __uint_as_float(0x3f800000u | (wa1 >> 9))), one);
+  const float2 ub = add2(make_float2(__uint_as_float(0x3f800000u | (wb0 >> 9)), __uint_as_float(0x3f800000u | (wb1 >> 9))), one);
+  const float2 ne = mul2(make_float2(lg2_approx(ua.x), lg2_approx(ua.y)), bc2(2.0f * kLn2F));  // 2 ln u
+  const float2 nr = mul2(ne, make_float2(rsqrt_approx(-ne.x), rsqrt_approx(-ne.y)));           // -sqrt(-2 ln u)
+  const float2 a = mul2(bc2(6.28318530717958647692f), add2(ub, bc2(-0.5f)));
+  z0 = mul2(nr, make_float2(cos_approx(a.x), cos_approx(a.y)));
+  z1 = mul2(nr, make_float2(sin_approx(a.x), sin_approx(a.y)));
 }
 
 // Register budget per particles-per-thread shape of the FP32 filter (grouped
@@ -275,21 +276,55 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
     for (int e = 0; e < NS; ++e) x[p][e] = make_float2(a[e], b[e]);
   }
 
-  // log p^(y_{1:t}) (Eq. 8) = lsum_m + lsum_hi + lsum_lo, carried by thread 0
+  // log p^(y_{1:t}) (Eq. 8) = lsum_m + lsum_hi + lsum_lo: the increments' maxima summed in FP64
+  // (exact for floats) and their brackets [(e - B) ln 2 + log(S 2^-e) - log M], a few units in size,
+  // as an unevaluated float pair (hi, lo) by Knuth's TwoSum, which keeps the sum to about 2^-48.
+  // At eight particles per thread lane (t - 1) % 32 of the first warp keeps step t's maximum and
+  // total, and every 32 steps the lanes take their brackets side by side and the sum runs over them
+  // in step order; below, where the three registers that takes would spill, thread 0 adds each step's.
+  constexpr bool DEFER = PPT == 8;
   double lsum_m = 0.0;
   float lsum_hi = 0.f, lsum_lo = 0.f;
+  float inc_m = 0.f;
+  uint64_t inc_S = 1;
   bool dead = false;
+  auto bracket = [&](uint64_t S) {
+    const int e = 63 - __clzll((long long)S);
+    const float mant = __uint2float_rn((uint32_t)(S >> (e - 31))) * 0x1p-31f;  // S / 2^e in [1, 2]
+    return fmaf((float)(e - B), (float)kLn2, logf(mant)) - logM;
+  };
+  auto add = [&](double m, float v) {
+    lsum_m += m;
+    const float sh = lsum_hi + v, bv = sh - lsum_hi;  // TwoSum: sh + err = lsum_hi + v exactly
+    lsum_lo += (lsum_hi - (sh - bv)) + (v - bv);
+    lsum_hi = sh;
+  };
+  auto add_increments = [&](int t_last) {  // the n = (t_last - 1) % 32 + 1 steps up to t_last
+    if (!DEFER || warp != 0 || t_last < 1) return;
+    const int n = ((t_last - 1) & 31) + 1;
+    const float small = bracket(inc_S);
+    const double md = (double)inc_m;
+    if constexpr (TRACE) {
+      if (J.delta && lane < n) J.delta[(size_t)i * J.T + (t_last - n) + lane] = md + (double)small;
+    }
+    for (int s = 0; s < n; ++s) add(__shfl_sync(0xffffffffu, md, s), __shfl_sync(0xffffffffu, small, s));
+  };
+  const bool ragged = M < Mp;
+  const float inv_M = 1.f / (float)M;
   for (int t = 1; t <= TT; ++t) {
+    if (((t - 1) & 31) == 0) add_increments(t - 1);
     const int tm = (t - 1) & 3;
     uint32_t* sUg = sU + 4 * (((t - 1) >> 2) & 1);
     if (tm == 0) {  // one Philox call per slot every four steps; the normals wait in shared memory
 #pragma unroll 1
       for (int p = 0; p < NP; ++p) {
-        float za[4], zb[4];
-        normals4_rk(make_uint4((uint32_t)(lt * PPT + 2 * p), (uint32_t)((t - 1) >> 2), c2, c3prop), rk, za);
-        normals4_rk(make_uint4((uint32_t)(lt * PPT + 2 * p + 1), (uint32_t)((t - 1) >> 2), c2, c3prop), rk, zb);
+        const uint4 wa = philox4x32_10_rk(make_uint4((uint32_t)(lt * PPT + 2 * p), (uint32_t)((t - 1) >> 2), c2, c3prop), rk);
+        const uint4 wb = philox4x32_10_rk(make_uint4((uint32_t)(lt * PPT + 2 * p + 1), (uint32_t)((t - 1) >> 2), c2, c3prop), rk);
+        float2 z[4];
+        box_muller2(wa.x, wb.x, wa.y, wb.y, z[0], z[1]);
+        box_muller2(wa.z, wb.z, wa.w, wb.w, z[2], z[3]);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) Z[(e * NP + p) * T + lt] = make_float2(za[e], zb[e]);
+        for (int e = 0; e < 4; ++e) Z[(e * NP + p) * T + lt] = z[e];
       }
       if (lt < 4 && t + lt < TT) sUg[lt] = philox4x32_10_rk(make_uint4(0u, (uint32_t)(t + lt), c2, c3res), rk).x;
       if (nw == 1) __syncwarp();  // the resampling words before the warp reads them (wider groups: barriers below)
@@ -304,8 +339,9 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
       float2 l2 = pm.step(x[p], Z[(tm * NP + p) * T + lt], ob, lam, dp, far);
       if (__any_sync(0xffffffffu, far != 0)) l2 = PairModel<MODEL>::fix_far(l2, dp, far, ob);  // rare
       const int j = lt * PPT + 2 * p;
-      const float la = (isnan(l2.x) || j >= M) ? -INFINITY : l2.x;
-      const float lb = (isnan(l2.y) || j + 1 >= M) ? -INFINITY : l2.y;
+      // -inf for a NaN and for the padding of the last threads
+      const float la = (ragged && j >= M) ? -INFINITY : fmaxf(l2.x, -INFINITY);
+      const float lb = (ragged && j + 1 >= M) ? -INFINITY : fmaxf(l2.y, -INFINITY);
       ell[2 * p] = la;
       ell[2 * p + 1] = lb;
       lmax = fmaxf(lmax, fmaxf(la, lb));
@@ -335,6 +371,7 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
     if (!(m > -INFINITY)) {  // every weight vanished: the estimate is zero
       dead = true;
       if constexpr (TRACE) {
+        if (((t - 1) & 31) != 0) add_increments(t - 1);
         if (lt == 0 && J.delta)
           for (int s = t; s <= J.T; ++s) J.delta[(size_t)i * J.T + (s - 1)] = -HUGE_VAL;
       }
@@ -380,19 +417,15 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
     } else {
       S = __shfl_sync(0xffffffffu, incl, 31);
     }
-    // (4) log-likelihood increment from the exact integer total (S >= 2^(B-1), B >= 51):
-    // max + [(e - B) ln 2 + log(S 2^-e) - log M].  The maxima are summed in FP64 (exact for
-    // floats); the bracket, a few units in size, as an unevaluated float pair (hi, lo) by
-    // Knuth's TwoSum, which keeps the sum to about 2^-48, so that a step costs the narrow
-    // FP64 pipe two instructions.
-    if (lt == 0) {
-      const int e = 63 - __clzll((long long)S);
-      const float mant = __uint2float_rn((uint32_t)(S >> (e - 31))) * 0x1p-31f;  // S / 2^e in [1, 2]
-      const float small = fmaf((float)(e - B), (float)kLn2, logf(mant)) - logM;
-      lsum_m += (double)m;
-      const float sh = lsum_hi + small, bv = sh - lsum_hi;  // TwoSum: sh + err = lsum_hi + small exactly
-      lsum_lo += (lsum_hi - (sh - bv)) + (small - bv);
-      lsum_hi = sh;
+    // (4) log-likelihood increment from the exact integer total (S >= 2^(B-1), B >= 51)
+    if (DEFER) {
+      if (warp == 0 && lane == ((t - 1) & 31)) {
+        inc_m = m;
+        inc_S = S;
+      }
+    } else if (lt == 0) {
+      const float small = bracket(S);
+      add((double)m, small);
       if constexpr (TRACE) {
         if (J.delta) J.delta[(size_t)i * J.T + (t - 1)] = (double)m + (double)small;
       }
@@ -405,7 +438,8 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
         fast_group_sync<GROUPED>(T, g);
       }
       const uint32_t tg = tag << kMarkBits;
-      const SlotCount sc = slot_count_setup(sUg[tm], S, M);
+      const uint32_t U = sUg[tm];
+      const SlotCount sc = slot_count_setup(U, S, M);
       const uint64_t C0 = base + excl;  // cumulative weight before the thread's first particle
       const float C0f = u64_to_float(C0);
       int ends[PPT + 1];
@@ -437,21 +471,21 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
         // float estimate (its error, under 17 M u, is far below 1/2), then
         // E = C0 M 2^33 - (2^33 n0 + 2U + 1) S, which is S 2^33 (x0 - n0) for the crossing
         // point x0 = C0 M / S - (2U + 1) 2^-33 of Eq. (27): F(C0) = n0 + [E > 0], and
-        // e0 = x0 - n0 = E 2^-33 / S to about 9 u.  |x0 - n0| < 1 and S <= 2^63 keep
+        // e0 = x0 - n0 = E 2^-33 / S to about 11 u.  |x0 - n0| < 1 and S <= 2^63 keep
         // E 2^-33 inside 64 bits.
         const int n0 = min(max((int)rintf(fmaf(C0f, sc.scale, -sc.off)), 0), M - 1);
-        const uint64_t a0 = ((uint64_t)n0 << 33) + sc.U21;
-        const uint64_t p_lo = a0 * sc.S, p_hi = __umul64hi(a0, sc.S);
-        const uint64_t q_lo = C0 * sc.M33, q_hi = __umul64hi(C0, sc.M33);
-        const uint64_t e_lo = q_lo - p_lo, e_hi = q_hi - p_hi - (q_lo < p_lo ? 1ull : 0ull);
-        const long long e33 = (long long)((e_hi << 31) | (e_lo >> 33));
-        const float e0 = fmaf((float)(int)(e33 >> 32), 0x1p32f, (float)(uint32_t)e33) * sc.scale / (float)M;
+        // floor((2U + 1) S / 2^33) from the 96-bit product U S; then E 2^-33 = C0 M - n0 S - (2U + 1) S 2^-33
+        // lies in (e33 - 1, e33], so E > 0 exactly when e33 >= 1 (all modulo 2^64)
+        const uint64_t us = (uint64_t)U * (uint32_t)S;
+        const uint64_t share = (uint64_t)U * (uint32_t)(S >> 32) + (us >> 32) + ((2ull * (uint32_t)us + S) >> 33);
+        const long long e33 = (long long)(C0 * (uint32_t)M - S * (uint32_t)n0 - share);
+        const float e0 = fmaf((float)(int)(e33 >> 32), 0x1p32f, (float)(uint32_t)e33) * (sc.scale * inv_M);
         // The later crossings x0 + s_r M / S, s_r the thread's share of the weight
         // before particle r: its float sum errs by 7 u of itself, M / S by 6 u and the
-        // product by 1 u, so y = e0 + s_r M / S errs by under 15 u s_r M / S + 10 u.  A
+        // product by 1 u, so y = e0 + s_r M / S errs by under 15 u s_r M / S + 12 u.  A
         // margin of 2^-19 (s_r M / S + 1) covers that twice; crossings inside it (rare:
         // the margin follows the share, not M) take the exact test.
-        ends[0] = n0 + (((long long)e_hi > 0 || (e_hi == 0 && e_lo != 0)) ? 1 : 0);
+        ends[0] = n0 + (e33 > 0 ? 1 : 0);
         uint32_t near_mask = 0;
 #pragma unroll
         for (int r = 1; r <= PPT; ++r) {
@@ -527,6 +561,7 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
       if (nw == 1) __syncwarp();  // every read done before the next step's writes
     }
   }
+  if (!dead) add_increments(TT);
   if (lt == 0) J.loglik[i] = dead ? -HUGE_VAL : lsum_m + ((double)lsum_hi + (double)lsum_lo);
 }
 

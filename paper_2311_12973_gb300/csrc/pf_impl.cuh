@@ -175,9 +175,9 @@ __device__ __forceinline__ double neg_inf<double>() {
 // two scaling; v - hi 2^32 = v mod 2^32 holds at most v's 24 significant bits), and
 // the two 32-bit conversions avoid the float-to-u64 one, which runs on the FP64 pipe.
 __device__ __forceinline__ uint64_t floor_to_u64(float v) {
-  const float hi = floorf(v * 0x1p-32f);
-  const float lo = fmaf(-hi, 0x1p32f, v);
-  return ((uint64_t)__float2uint_rz(hi) << 32) | (uint64_t)__float2uint_rz(lo);
+  const uint32_t hi = __float2uint_rz(v * 0x1p-32f);
+  const float lo = fmaf(-__uint2float_rn(hi), 0x1p32f, v);
+  return ((uint64_t)hi << 32) | (uint64_t)__float2uint_rz(lo);
 }
 
 // u64 to float from its two 32-bit halves (relative error below 2^-23).
