@@ -1146,8 +1146,8 @@ smc2_status smc2_mlp_adam_step(int D, float* params, float* m, float* v, int* st
       !(lr >= 0.f && lr < 1.f))
     return SMC2_EINVAL;
   if (reinterpret_cast<uintptr_t>(params) % 16 != 0) return SMC2_EINVAL;  // the documented layout
-  SMC2_TRY(mlp_train_steps_launch(params, m, v, step, const_cast<float*>(x), const_cast<float*>(y), R, nullptr,
-                                  loss, D, 1, lr, static_cast<cudaStream_t>(stream)));
+  SMC2_TRY(mlp_train_steps_launch(params, m, v, step, const_cast<float*>(x), const_cast<float*>(y), R, loss,
+                                  D, 1, lr, static_cast<cudaStream_t>(stream)));
   return SMC2_OK;
 }
 
@@ -1158,23 +1158,8 @@ smc2_status smc2_mlp_train_ring(int D, float* params, float* m, float* v, int* s
       !ring_lp || !x || !y || !stdz || !(lr >= 0.f && lr < 1.f))
     return SMC2_EINVAL;
   if (reinterpret_cast<uintptr_t>(params) % 16 != 0) return SMC2_EINVAL;  // the documented layout
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  struct Scratch {
-    MlpNorm nm;
-    float loss;
-    int rows;
-  };
-  Scratch* w = nullptr;
-  SMC2_TRY(cudaMallocAsync(reinterpret_cast<void**>(&w), sizeof(Scratch), s));
-  cudaError_t e = cudaMemsetAsync(w, 0, sizeof(Scratch), s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&w->rows, &R, sizeof(int), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess)
-    e = mlp_train_ring_launch(params, m, v, step, ring_th, ring_lp, &w->rows, R, &w->nm, x, y, &w->loss, D, steps,
-                              lr, s);
-  if (e == cudaSuccess) e = mlp_norm_export_launch(&w->nm, &w->loss, D, stdz, s);
-  const cudaError_t ef = cudaFreeAsync(w, s);
-  SMC2_TRY(e);
-  SMC2_TRY(ef);
+  SMC2_TRY(mlp_train_ring_launch(params, m, v, step, ring_th, ring_lp, R, x, y, stdz, D, steps, lr,
+                                 static_cast<cudaStream_t>(stream)));
   return SMC2_OK;
 }
 

@@ -209,22 +209,17 @@ cudaError_t resample_systematic_launch(const uint64_t* q, int n, uint32_t U, int
 // Surrogate network (mlp.cu).
 int mlp_param_count(int D);
 int mlp_grad_ctas(int R);  // CTAs (and partial-gradient rows) of one training step over R rows
-size_t mlp_grad_smem_bytes();
 cudaError_t mlp_step_launch(float* p, int D, const float* x, const float* y, int R, const int* R_dev,
                             float* part, float* grad, float* loss, int adam, float* m, float* v, int* step,
                             float lr, cudaStream_t s);
 int mlp_train_cluster_size();  // CTAs of the training cluster (0: no cluster can be scheduled)
-size_t mlp_train_smem_bytes();
 // Per-SM footprint of the training cluster: its CTAs, and one CTA's threads,
 // registers per thread and shared memory.
 cudaError_t mlp_train_footprint(int* ctas, int* threads, int* regs, size_t* smem);
-cudaError_t mlp_train_steps_launch(float* p, float* m, float* v, int* step, float* x, float* y, int R,
-                                   const int* R_dev, float* loss, int D, int steps, float lr, cudaStream_t s,
-                                   const MlpDev* ring_of = nullptr);
-cudaError_t mlp_train_ring_launch(float* p, float* m, float* v, int* step, const float* th, const float* lp,
-                                  const int* rows_dev, int R, MlpNorm* norm, float* x, float* y, float* loss,
-                                  int D, int steps, float lr, cudaStream_t s);
-cudaError_t mlp_norm_export_launch(const MlpNorm* nm, const float* loss, int D, double* out, cudaStream_t s);
+cudaError_t mlp_train_steps_launch(float* p, float* m, float* v, int* step, float* x, float* y, int R, float* loss,
+                                   int D, int steps, float lr, cudaStream_t s);
+cudaError_t mlp_train_ring_launch(float* p, float* m, float* v, int* step, const float* th, const float* lp, int R,
+                                  float* x, float* y, double* stdz, int D, int steps, float lr, cudaStream_t s);
 cudaError_t mlp_init_launch(const MlpDev& M, int D, uint64_t seed, cudaStream_t s);
 cudaError_t mlp_append_launch(const OuterParams& P, int N, cudaStream_t s);
 cudaError_t mlp_train_launch(const OuterParams& P, int steps, float lr, cudaStream_t s);
