@@ -240,6 +240,17 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
   // dataset's layout, and the step tag restarts at 1
   for (int s = lt; s < Mp; s += T) mark[s] = 0u;
   carry[lt] = 0u;  // threads whose slots are all padding keep this valid ancestor (particle 0)
+  // With four or eight particles per thread, a group of up to eight warps reads its warps' maxima and
+  // totals as vectors (every thread the same words) and combines them itself, which is shorter than the
+  // reduction and the scan over the lanes that other groups take: four warps, N=1024/M=512/T=100 at ppt 4
+  // 374 -> 357 us and N=8192/M=1024/T=200 at ppt 8 9.65 -> 9.38 ms; eight warps, N=200/M=1000/T=100 at
+  // ppt 4 271 -> 265 us.  (At two particles per thread it measured 0 to 3 % slower.)  Warps that the group
+  // lacks count for nothing.
+  constexpr bool kVec = PPT >= 4;
+  if (kVec && lt < 8) {
+    wmax[lt] = -INFINITY;
+    wsum[lt] = 0ull;
+  }
   uint32_t tag = 0;
   fast_group_sync<GROUPED>(T, g);
 
@@ -362,10 +373,18 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
     }
     // (2) group maximum
     lmax = warp_max_redux(lmax);
-    if (nw > 1) {  // lane w reads warp w's maximum; one more reduction spreads the group's
+    if (nw > 1) {  // in a wide group lane w reads warp w's maximum; one more reduction spreads the group's
       if (lane == 0) wmax[warp] = lmax;
       fast_group_sync<GROUPED>(T, g);
-      lmax = warp_max_redux(lane < nw ? wmax[lane] : -INFINITY);
+      if (kVec && nw <= 4) {
+        const float4 wm = *reinterpret_cast<const float4*>(wmax);
+        lmax = fmaxf(fmaxf(wm.x, wm.y), fmaxf(wm.z, wm.w));
+      } else if (kVec && nw <= 8) {
+        const float4 wm = *reinterpret_cast<const float4*>(wmax), wn = *reinterpret_cast<const float4*>(wmax + 4);
+        lmax = fmaxf(fmaxf(fmaxf(wm.x, wm.y), fmaxf(wm.z, wm.w)), fmaxf(fmaxf(wn.x, wn.y), fmaxf(wn.z, wn.w)));
+      } else {
+        lmax = warp_max_redux(lane < nw ? wmax[lane] : -INFINITY);
+      }
     }
     const float m = lmax;
     if (!(m > -INFINITY)) {  // every weight vanished: the estimate is zero
@@ -403,17 +422,32 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
     const uint64_t incl = warp_incl_scan_u64(run, lane);
     const uint64_t excl = incl - run;
     uint64_t S, base = 0;
-    if (nw > 1) {  // lane w reads warp w's total; an inclusive shuffle scan gives S and the warp's base
+    if (nw > 1) {  // in a wide group lane w reads warp w's total; an inclusive shuffle scan gives S and the warp's base
       if (lane == 31) wsum[warp] = incl;
       fast_group_sync<GROUPED>(T, g);
-      uint64_t wp = lane < nw ? wsum[lane] : 0ull;
-      for (int o = 1; o < nw; o <<= 1) {
-        const uint64_t n = __shfl_up_sync(0xffffffffu, wp, o);
-        if (lane >= o) wp += n;
+      if (kVec && nw <= 4) {
+        const ulonglong2 w01 = *reinterpret_cast<const ulonglong2*>(wsum);
+        const ulonglong2 w23 = *reinterpret_cast<const ulonglong2*>(wsum + 2);
+        const uint64_t p2 = w01.x + w01.y, p3 = p2 + w23.x;
+        S = p3 + w23.y;
+        base = warp == 0 ? 0ull : (warp == 1 ? w01.x : (warp == 2 ? p2 : p3));
+      } else if (kVec && nw <= 8) {
+        const ulonglong2* v = reinterpret_cast<const ulonglong2*>(wsum);
+        const ulonglong2 w01 = v[0], w23 = v[1], w45 = v[2], w67 = v[3];
+        const uint64_t p2 = w01.x + w01.y, p4 = p2 + (w23.x + w23.y), p6 = p4 + (w45.x + w45.y);
+        S = p6 + (w67.x + w67.y);
+        base = (warp & 4) ? ((warp & 2) ? p6 : p4) : ((warp & 2) ? p2 : 0ull);
+        if (warp & 1) base += (warp & 4) ? ((warp & 2) ? w67.x : w45.x) : ((warp & 2) ? w23.x : w01.x);
+      } else {
+        uint64_t wp = lane < nw ? wsum[lane] : 0ull;
+        for (int o = 1; o < nw; o <<= 1) {
+          const uint64_t n = __shfl_up_sync(0xffffffffu, wp, o);
+          if (lane >= o) wp += n;
+        }
+        S = __shfl_sync(0xffffffffu, wp, nw - 1);
+        const uint64_t b = __shfl_sync(0xffffffffu, wp, warp > 0 ? warp - 1 : 0);
+        base = warp > 0 ? b : 0ull;
       }
-      S = __shfl_sync(0xffffffffu, wp, nw - 1);
-      const uint64_t b = __shfl_sync(0xffffffffu, wp, warp > 0 ? warp - 1 : 0);
-      base = warp > 0 ? b : 0ull;
     } else {
       S = __shfl_sync(0xffffffffu, incl, 31);
     }

@@ -1299,7 +1299,15 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
     lmax = warp_max_num(lmax);
     if (nw > 1 && lane == 0) wmax[warp] = lmax;
     group_sync();
-    if (nw > 1) lmax = warp_max_num(lane < nw ? wmax[lane] : neg_inf<double>());
+    // Up to four warps' maxima and totals are combined by every thread from the same words, which is
+    // shorter than the reduction and the scan over the lanes that more warps take: where one particle per
+    // thread leaves each step to latency (LG run, N=64/M=128/T=50/K=10: 1.397 -> 1.369 ms; with more
+    // particles per thread no difference)
+    const bool few = PPT == 1 && nw <= 4;
+    if (few)
+      lmax = nw > 1 ? max_num(max_num(wmax[0], wmax[1]), max_num(wmax[nw > 2 ? 2 : 0], wmax[nw > 3 ? 3 : 0])) : lmax;
+    else if (nw > 1)
+      lmax = warp_max_num(lane < nw ? wmax[lane] : neg_inf<double>());
     const double m = lmax;
     if (m == neg_inf<double>()) {  // every weight vanished: the estimate is zero
       if (((t - 1) & 31) != 0) add_increments(t - 1);
@@ -1325,14 +1333,21 @@ __device__ __forceinline__ void run_filter64(const PFJob& J, const PFModel& mdl,
     if (adaptive) store_q2_float<PPT>(c, lane, reinterpret_cast<float*>(wq2 + warp));
     group_sync();
     // total S, and the weight `base` of the warps before this one
-    uint64_t wpre = lane < nw ? wsum[lane] : 0ull;
-    for (int o = 1; o < nw; o <<= 1) {
-      const uint64_t n = __shfl_up_sync(0xffffffffu, wpre, o);
-      if (lane >= o) wpre += n;
+    uint64_t S, C0 = excl;  // C0: weight before the thread's first particle
+    if (few) {
+      const uint64_t w0 = wsum[0], p2 = w0 + (nw > 1 ? wsum[1] : 0ull), p3 = p2 + (nw > 2 ? wsum[2] : 0ull);
+      S = p3 + (nw > 3 ? wsum[3] : 0ull);
+      C0 += warp == 0 ? 0ull : (warp == 1 ? w0 : (warp == 2 ? p2 : p3));
+    } else {
+      uint64_t wpre = lane < nw ? wsum[lane] : 0ull;
+      for (int o = 1; o < nw; o <<= 1) {
+        const uint64_t n = __shfl_up_sync(0xffffffffu, wpre, o);
+        if (lane >= o) wpre += n;
+      }
+      S = __shfl_sync(0xffffffffu, wpre, nw - 1);
+      const uint64_t base_incl = __shfl_sync(0xffffffffu, wpre, warp > 0 ? warp - 1 : 0);
+      C0 += warp > 0 ? base_incl : 0ull;
     }
-    const uint64_t S = __shfl_sync(0xffffffffu, wpre, nw - 1);
-    const uint64_t base_incl = __shfl_sync(0xffffffffu, wpre, warp > 0 ? warp - 1 : 0);
-    const uint64_t C0 = (warp > 0 ? base_incl : 0ull) + excl;  // weight before the thread's first particle
     // (5) likelihood increment (Eq. 8): see add_increments
     const bool mine = lane == ((t - 1) & 31);
     inc_m = mine ? m : inc_m;
