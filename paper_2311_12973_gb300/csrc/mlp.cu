@@ -4,9 +4,9 @@
 // bfloat16 operands and FP32 accumulation (mma.sync m16n8k16).  A warp owns
 // 16 rows; the accumulator fragments of one layer are re-packed in registers
 // as the operand fragments of the next.  Training computes per-CTA partial
-// gradients of the mean squared error (the weight gradient dW2 = h1^T dz2 is
-// a second product over the CTA's 64 rows, staged transposed in shared
-// memory), then one kernel sums them in a fixed order and takes an Adam step.
+// gradients of the mean squared error (the weight gradients are second products
+// over the CTA's rows, staged in shared memory) and sums them in a fixed order
+// for an Adam step.
 // The proposal uses the gradient with respect to the input.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>

@@ -27,7 +27,7 @@
 //      after a barrier the ancestor of slot s is the largest current tag at or
 //      before s within its thread's slots -- ancestors never decrease along the
 //      slots -- and the thread reads that particle's state.
-// The step is bound by instruction issue (about 60 % of the slots; the rest waits on fixed
+// The step is bound by instruction issue (64 % of the slots; the rest waits on fixed
 // latencies and the three barriers).  What an instruction count bought last, same results bit for
 // bit: approximations without subnormal handling, packed Box-Muller, one fmaxf for NaN and the
 // first crossing's exact test from 64-by-32-bit products (6 wide multiplies where the 128-bit
