@@ -66,7 +66,7 @@ struct smc2_ctx {
   cudaStream_t stream = nullptr, cap_stream = nullptr, side_stream = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaStream_t train_stream = nullptr;              // learned-proposal training branch
-  cudaEvent_t ev_tfork = nullptr, ev_tjoin = nullptr;
+  cudaEvent_t ev_tfork = nullptr, ev_append = nullptr, ev_publish = nullptr, ev_tjoin = nullptr;
   bool train_pending = false;                       // while capturing: branch not yet joined
   int device = 0, sms = 0;
   char* arena = nullptr;
@@ -618,17 +618,24 @@ smc2_status enqueue_iteration(smc2_ctx* c, cudaStream_t s, cudaEvent_t ev0, cuda
   SMC2_TRY(cudaStreamWaitEvent(s, c->ev_join, 0));
   SMC2_TRY(outer_weights(c->op, c->max_nblk, s));
   if (c->mlp.on) {
-    SMC2_TRY(join_training(c, s));
-    SMC2_TRY(mlp_publish_launch(c->op, s));
-    SMC2_TRY(mlp_append_launch(c->op, c->N[0], s));
+    // On the training stream, behind the last call's training: this iteration's rows are stored (before the
+    // resampling advances the iteration), the trained state is published (before the next score reads it),
+    // and the next training starts.  The main stream quantises beside the first two (a run of N=1024/M=512/
+    // T=100/K=20: 9.65 -> 9.50 ms).
     SMC2_TRY(cudaEventRecord(c->ev_tfork, s));
     SMC2_TRY(cudaStreamWaitEvent(c->train_stream, c->ev_tfork, 0));
+    SMC2_TRY(mlp_append_launch(c->op, c->N[0], c->train_stream));
+    SMC2_TRY(cudaEventRecord(c->ev_append, c->train_stream));
+    SMC2_TRY(mlp_publish_launch(c->op, c->train_stream));
+    SMC2_TRY(cudaEventRecord(c->ev_publish, c->train_stream));
     SMC2_TRY(mlp_train_launch(c->op, c->cfg.mlp_steps, (float)c->cfg.mlp_lr, c->train_stream));
     SMC2_TRY(cudaEventRecord(c->ev_tjoin, c->train_stream));
     c->train_pending = true;
   }
   SMC2_TRY(outer_quantise(c->op, c->max_nblk, s));
+  if (c->mlp.on) SMC2_TRY(cudaStreamWaitEvent(s, c->ev_append, 0));
   SMC2_TRY(outer_resample(c->op, c->max_nblk_res, c->max_N, s));
+  if (c->mlp.on) SMC2_TRY(cudaStreamWaitEvent(s, c->ev_publish, 0));
   return SMC2_OK;
 }
 
@@ -779,6 +786,8 @@ smc2_status smc2_init(const smc2_config* cfg, const double* y, void* stream, smc
       cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess ||
       cudaStreamCreateWithFlags(&c->train_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_tfork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_append, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_publish, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_tjoin, cudaEventDisableTiming) != cudaSuccess)
     return fail(SMC2_ECUDA);
 
@@ -1227,6 +1236,8 @@ void smc2_destroy(smc2_ctx* c) {
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->train_stream) cudaStreamDestroy(c->train_stream);
   if (c->ev_tfork) cudaEventDestroy(c->ev_tfork);
+  if (c->ev_append) cudaEventDestroy(c->ev_append);
+  if (c->ev_publish) cudaEventDestroy(c->ev_publish);
   if (c->ev_tjoin) cudaEventDestroy(c->ev_tjoin);
   delete c;
 }
