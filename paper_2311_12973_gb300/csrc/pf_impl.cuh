@@ -416,8 +416,11 @@ struct FilterParams<double, MODEL_SEIR> {
     I0 = m.i0;
     c_m = s64_unpack(dt / m.npop, c_e);
     k_m = s64_unpack(kdt, k_e);
-    // no product overflows or underflows within a day: npop, kappa dt and gamma dt are moderate
-    tame = m.npop > 0x1p-20 && m.npop < 0x1p60 && kdt > 0x1p-100 && kdt < 0x1p20 && gdt < 0x1p20;
+    // no product overflows or underflows within a day: npop, kappa dt and gamma dt are moderate, and S,
+    // which stays non-negative and never grows, starts so (the allocation-free entry point takes
+    // e0 + i0 > npop, and s64_unpack wants no sign)
+    tame = m.npop > 0x1p-20 && m.npop < 0x1p60 && kdt > 0x1p-100 && kdt < 0x1p20 && gdt < 0x1p20 &&
+           S0 >= 0.0 && S0 < 0x1p61;
   }
   __device__ __forceinline__ void init(double* x, double, const double*) const {
     x[0] = S0;
