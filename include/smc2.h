@@ -28,6 +28,11 @@
  *    hardware barriers) and compute every index they use from exact integer
  *    arithmetic on validated sizes, so no device status exists for an expired
  *    wait or an index out of range.
+ *  - Host threads: calls that read a context (smc2_estimate, smc2_get_history,
+ *    smc2_get_proposals, smc2_get_learned_state, smc2_get_learned_training,
+ *    smc2_get_state, smc2_sync) may run on several threads at once and beside
+ *    one smc2_run or smc2_iterate.  No other two calls on one context may
+ *    overlap.
  *  - Parameters theta are in unconstrained coordinates:
  *      SMC2_MODEL_LG_AR1: (phi, log sigma_x, log sigma_y), D = 3;
  *      SMC2_MODEL_SEIR:   (log beta0, log sigma_rw, log kappa, log gamma), D = 4.

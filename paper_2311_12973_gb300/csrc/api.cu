@@ -4,10 +4,12 @@
 // build the particle-filter work list, enqueue kernels on the context stream
 // and capture iterations into CUDA graphs.  No step of the sampler runs here.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -81,14 +83,15 @@ struct smc2_ctx {
   int* d_wu_counter = nullptr;
   int* d_k = nullptr;
   int* d_status = nullptr;
-  char* pinned = nullptr;   // page-locked staging of read-backs (kPinnedBytes)
+  char* pinned = nullptr;   // page-locked staging of read-backs (kPinnedBytes), held by one read-back at a time
+  std::mutex pinned_mutex;
   unsigned* d_grid_ticket = nullptr;
   int ppt = 4, pf_block = 256, pf_grid = 1;
   bool pf_named = false;    // pf_kernel: named-barrier groups; the FP32 filter: grouped instantiation
   bool pf_general = false;  // the paper's PF variants: multinomial slots, ESS-triggered resampling
   bool pf_fast = false;     // the FP32 filter of pf_fast.cuh runs
   size_t pf_smem = 0;
-  int k_host = 0;
+  std::atomic<int> k_host{0};  // iterations enqueued (read by other threads' calls)
   std::map<GraphKey, TimedGraph> graphs;
   bool timing = false;
   double pf_ms = 0.0;
@@ -687,9 +690,11 @@ void drop_graphs(smc2_ctx* c) {
 }
 
 // The pieces of one read-back: device ranges copied to host places, then one wait and the sticky
-// device status.
+// device status.  It holds the context's staging buffer from its construction to its end, so that
+// several host threads may read one context (each then waits for the stream in turn).
 struct ReadBack {
   smc2_ctx* c;
+  std::lock_guard<std::mutex> hold;
   struct Piece {
     void* dst;
     const char* staged;
@@ -697,7 +702,7 @@ struct ReadBack {
   };
   std::vector<Piece> pieces;
   size_t used = sizeof(double);  // the status word leads the buffer
-  explicit ReadBack(smc2_ctx* ctx) : c(ctx) {}
+  explicit ReadBack(smc2_ctx* ctx) : c(ctx), hold(ctx->pinned_mutex) {}
   cudaError_t add(void* dst, const void* src, size_t bytes) {
     if (!dst || !bytes) return cudaSuccess;
     if (used + bytes > kPinnedBytes) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, c->stream);
@@ -964,13 +969,14 @@ smc2_status smc2_iterate(smc2_ctx* c, smc2_iter_stats* stats_host) {
 smc2_status smc2_estimate(smc2_ctx* c, int dataset, double* mean_host, double* logz_host,
                           double* ess_sum_host, double* cov_host) {
   if (bad_ds(c, dataset)) return SMC2_EINVAL;
-  if (c->k_host < 1) return SMC2_ESTATE;
+  const int k = c->k_host;
+  if (k < 1) return SMC2_ESTATE;
   const DSDev& s = c->h_ds[dataset];
   const int D = c->D;
   smc2_iter_stats last;
   std::vector<double> rec((size_t)1 + D + D * D);
   ReadBack rb(c);
-  SMC2_TRY(rb.add(&last, s.hist + (c->k_host - 1), sizeof(last)));
+  SMC2_TRY(rb.add(&last, s.hist + (k - 1), sizeof(last)));
   SMC2_TRY(rb.add(rec.data(), s.rec, rec.size() * sizeof(double)));
   const smc2_status st = rb.finish();
   const double l = rec[0];
@@ -988,11 +994,11 @@ smc2_status smc2_estimate(smc2_ctx* c, int dataset, double* mean_host, double* l
 
 smc2_status smc2_get_history(smc2_ctx* c, int dataset, smc2_iter_stats* hist, int cap, int* k_out) {
   if (bad_ds(c, dataset) || !hist || cap < 0) return SMC2_EINVAL;
-  const int k = std::min(c->k_host, cap);
+  const int k_all = c->k_host, k = std::min(k_all, cap);
   if (k > 0)
     SMC2_TRY(cudaMemcpyAsync(hist, c->h_ds[dataset].hist, (size_t)k * sizeof(smc2_iter_stats),
                              cudaMemcpyDeviceToHost, c->stream));
-  if (k_out) *k_out = c->k_host;
+  if (k_out) *k_out = k_all;
   return sticky(c);
 }
 
