@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -700,21 +701,28 @@ struct ReadBack {
     const char* staged;
     size_t bytes;
   };
-  std::vector<Piece> pieces;
-  size_t used = sizeof(double);  // the status word leads the buffer
+  Piece pieces[4];  // no call reads more (and no allocation can throw)
+  int n_pieces = 0;
+  size_t used = 16;  // the status word leads the buffer
   explicit ReadBack(smc2_ctx* ctx) : c(ctx), hold(ctx->pinned_mutex) {}
-  cudaError_t add(void* dst, const void* src, size_t bytes) {
-    if (!dst || !bytes) return cudaSuccess;
-    if (used + bytes > kPinnedBytes) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, c->stream);
+  static bool fits(size_t bytes, size_t used = 16) { return used + bytes <= kPinnedBytes; }
+  char* take(size_t bytes) {  // room for a piece that fits
     char* at = c->pinned + used;
     used += (bytes + 15) & ~(size_t)15;
-    pieces.push_back({dst, at, bytes});
+    return at;
+  }
+  cudaError_t add(void* dst, const void* src, size_t bytes) {
+    if (!dst || !bytes) return cudaSuccess;
+    if (!fits(bytes, used) || n_pieces == 4)
+      return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, c->stream);
+    char* at = take(bytes);
+    pieces[n_pieces++] = {dst, at, bytes};
     return cudaMemcpyAsync(at, src, bytes, cudaMemcpyDeviceToHost, c->stream);
   }
   smc2_status finish() {
     SMC2_TRY(cudaMemcpyAsync(c->pinned, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     SMC2_TRY(cudaStreamSynchronize(c->stream));
-    for (const Piece& p : pieces) memcpy(p.dst, p.staged, p.bytes);
+    for (int i = 0; i < n_pieces; ++i) memcpy(pieces[i].dst, pieces[i].staged, pieces[i].bytes);
     int bits = 0;
     memcpy(&bits, c->pinned, sizeof(int));
     return status_from_bits(bits);
@@ -929,6 +937,14 @@ smc2_status smc2_run(smc2_ctx* c, int n_iter, smc2_iter_stats* stats_host) {
   const TraceRange range("smc2_run");
   if (!c || n_iter < 1) return SMC2_EINVAL;
   if (c->k_host + n_iter > c->K) return SMC2_ESTATE;
+  // several datasets' statistics arrive dataset-major, as on the device: in the staging buffer, or when they
+  // exceed it in an array that is there before anything runs
+  const size_t n_stats = (size_t)c->n_ds * n_iter;
+  std::unique_ptr<smc2_iter_stats[]> by_dataset;
+  if (stats_host && c->n_ds > 1 && !ReadBack::fits(n_stats * sizeof(smc2_iter_stats))) {
+    by_dataset.reset(new (std::nothrow) smc2_iter_stats[n_stats]);
+    if (!by_dataset) return SMC2_ENOMEM;
+  }
   TimedGraph* g = nullptr;
   smc2_status st = get_graph(c, n_iter, &g);
   if (st != SMC2_OK) return st;
@@ -951,9 +967,11 @@ smc2_status smc2_run(smc2_ctx* c, int n_iter, smc2_iter_stats* stats_host) {
       SMC2_TRY(rb.add(stats_host, c->h_ds[0].hist + k0, (size_t)n_iter * sizeof(smc2_iter_stats)));
       return rb.finish();
     }
-    std::vector<smc2_iter_stats> h((size_t)c->n_ds * n_iter);  // dataset-major, as on the device
+    smc2_iter_stats* h = by_dataset ? by_dataset.get()
+                                    : reinterpret_cast<smc2_iter_stats*>(rb.take(n_stats * sizeof(smc2_iter_stats)));
     for (int d = 0; d < c->n_ds; ++d)
-      SMC2_TRY(rb.add(h.data() + (size_t)d * n_iter, c->h_ds[d].hist + k0, (size_t)n_iter * sizeof(smc2_iter_stats)));
+      SMC2_TRY(cudaMemcpyAsync(h + (size_t)d * n_iter, c->h_ds[d].hist + k0, (size_t)n_iter * sizeof(smc2_iter_stats),
+                               cudaMemcpyDeviceToHost, c->stream));
     const smc2_status done = rb.finish();
     for (int d = 0; d < c->n_ds; ++d)
       for (int i = 0; i < n_iter; ++i) stats_host[(size_t)i * c->n_ds + d] = h[(size_t)d * n_iter + i];
