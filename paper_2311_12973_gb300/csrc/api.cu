@@ -909,8 +909,17 @@ static smc2_status pf_standalone(smc2_ctx* c, const double* theta, int n, int it
   }
   const int occ = std::max(1, ctx_pf_occupancy(c, trace));
   const int grid = std::min(L.n_wu, occ * c->sms);
-  // more units than fit at once: from the queue, so that CTAs with light filters take more of them
-  if (L.n_wu > grid) L.wu_counter = c->d_wu_counter;
+  // more units than fit at once: from the queue, so that CTAs with light filters take more of them.  The queue
+  // is the context's one, which its stream's order protects; a captured launch may be replayed on any stream,
+  // beside the context's work or another replay, and keeps the static split.
+  if (L.n_wu > grid) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(c->stream, &capture) != cudaSuccess) {
+      capture = cudaStreamCaptureStatusActive;
+      cudaGetLastError();
+    }
+    if (capture == cudaStreamCaptureStatusNone) L.wu_counter = c->d_wu_counter;
+  }
   SMC2_TRY(ctx_pf_launch(c, grid, L, c->stream, trace));
   c->kernel_launches++;
   return SMC2_OK;
