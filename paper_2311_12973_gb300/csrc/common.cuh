@@ -167,16 +167,28 @@ __device__ __forceinline__ int fixed_point_bits(int n) {
 }
 
 // floor((2^33 j + 2U + 1) S / (n 2^33)): the threshold of slot j < n < 2^15.  The shift by 33
-// comes first (floors nest), which leaves less than 2^78; the division by n then takes two steps
-// of 64 by 32 bits in place of a general 128-bit one.
-__device__ __forceinline__ uint64_t slot_threshold(uint32_t j, uint32_t U, uint64_t S, int n,
-                                                   int log2n) {
+// comes first (floors nest), which leaves less than 2^79; the division by n then takes two steps
+// of at most 47 bits by n, each a high product with inv = slot_reciprocal(n) and one correction
+// (inv falls short of 2^64 / n by at most 1 + 1/n, so a quotient is at most one too small).  A
+// filter or a block forms inv once.  The staged filters (ppt 8 and 16) take a threshold for every
+// slot in unrolled code: mixed precision, LG N=231/M=900/T=50 at ppt 8, 492 us with a 128-bit
+// division, 577 with two general 64-bit ones, 384 so; FP64 896 with those, 712 so.  A power of two
+// needs only the shift (N=600/M=128/T=50: 306 us, 318 with the products).
+__device__ __forceinline__ uint64_t slot_reciprocal(int n) { return ~0ull / (uint32_t)n; }
+__device__ __forceinline__ uint64_t slot_threshold(uint32_t j, uint32_t U, uint64_t S, int n, uint64_t inv) {
   const unsigned __int128 num = (((unsigned __int128)j << 33) + 2ull * U + 1ull) * S;
-  if (log2n >= 0) return (uint64_t)(num >> (33 + log2n));
+  if ((n & (n - 1)) == 0) return (uint64_t)(num >> (32 + __ffs(n)));
   const unsigned __int128 a = num >> 33;
-  const uint64_t top = (uint64_t)(a >> 32), q1 = top / (uint32_t)n;
-  const uint64_t low = ((top - q1 * (uint32_t)n) << 32) | (uint32_t)a;
-  return (q1 << 32) + low / (uint32_t)n;
+  const uint32_t d = (uint32_t)n;
+  const uint64_t top = (uint64_t)(a >> 32);
+  uint64_t q1 = __umul64hi(top, inv), rest = top - q1 * d;
+  if (rest >= d) {
+    ++q1;
+    rest -= d;
+  }
+  const uint64_t low = (rest << 32) | (uint32_t)a;
+  const uint64_t q2 = __umul64hi(low, inv);
+  return (q1 << 32) + q2 + (low - q2 * d >= d ? 1u : 0u);
 }
 
 template <typename R>

@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(kOuterBlock) quantise_kernel(OuterParams P) {
 // its run as prefixes.  Runs have odd length, so that the lanes' 8-byte accesses fall into
 // different banks.  Four barriers whatever n is.  The primitive at n = 10007, whole call: 20.5 us
 // with a scan of 256 entries at a time (two barriers for each) and a general 128-bit division per
-// slot, 8.2 us with this one and slot_threshold's two short divisions.
+// slot, 8.5 us with this one and two 64-bit divisions, 7.6 us with slot_threshold's high products (runs differ by 10 %).
 __device__ uint64_t scan_all_to_smem(const uint64_t* q, int n, uint64_t* C) {
   __shared__ uint64_t wt[kResWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -611,9 +611,8 @@ __global__ void __launch_bounds__(kResBlock) resample_kernel(OuterParams P) {
       const uint64_t total = scan_all_to_smem(S.q, N, C);
       const uint32_t U =
           philox4x32_10(make_uint4(0u, 0u, S.c2hi, counter_c3(TAG_OUTER_RES, k)), seed_key(P.seed)).x;
-      const int log2n = ((N & (N - 1)) == 0) ? (__ffs(N) - 1) : -1;
       if (j < N) {
-        const uint64_t tau = slot_threshold((uint32_t)j, U, total, N, log2n);
+        const uint64_t tau = slot_threshold((uint32_t)j, U, total, N, slot_reciprocal(N));
         const int a = search_first_greater(C, N, tau);
         for (int d = 0; d < D; ++d) S.thA[(size_t)d * N + j] = S.thB[(size_t)d * N + a];
         S.lpA[j] = S.lpB[a];
@@ -643,9 +642,8 @@ __global__ void __launch_bounds__(kResBlock)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint64_t* C = reinterpret_cast<uint64_t*>(smem_raw);
   const uint64_t total = scan_all_to_smem(q, n, C);
-  const int log2n = ((n & (n - 1)) == 0) ? (__ffs(n) - 1) : -1;
   const int j = blockIdx.x * kResBlock + threadIdx.x;
-  if (j < n && total > 0) anc[j] = search_first_greater(C, n, slot_threshold((uint32_t)j, U, total, n, log2n));
+  if (j < n && total > 0) anc[j] = search_first_greater(C, n, slot_threshold((uint32_t)j, U, total, n, slot_reciprocal(n)));
 }
 
 __global__ void philox_normals_kernel(uint64_t seed, const uint32_t* ctr, int n, int precision,

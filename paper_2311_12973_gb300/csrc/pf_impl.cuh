@@ -769,7 +769,7 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
   const uint32_t c3multi = counter_c3(TAG_PF_MULTI, k);
   const uint32_t c3binom = counter_c3(TAG_PF_BINOM, k);
   const int B = fixed_point_bits(M);
-  const int log2M = ((M & (M - 1)) == 0) ? (__ffs(M) - 1) : -1;
+  const uint64_t inv_M = STAGED ? slot_reciprocal(M) : 0ull;
   const R scaleB = (R)ldexp(1.0, B);
   const double log_norm = warp == 0 ? -(double)B * kLn2 - log((double)M) : 0.0;  // thread 0's
   const R4* obs = reinterpret_cast<const R4*>(J.obs);
@@ -1054,7 +1054,7 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
       for (int r = 0; r < PPT; ++r) {
         const int j = lt * PPT + r;
         if (j < M) {
-          const uint64_t tau = slot_threshold((uint32_t)j, U, S, M, log2M);
+          const uint64_t tau = slot_threshold((uint32_t)j, U, S, M, inv_M);
           while (w < nw - 1 && base + wsum[w] <= tau) {  // answer lies in a later warp
             base += wsum[w];
             ++w;
