@@ -297,7 +297,7 @@ __device__ __forceinline__ void fast_filter(const PFJob& J, const PFModel& mdl, 
   double lsum_m = 0.0;
   float lsum_hi = 0.f, lsum_lo = 0.f;
   float inc_m = 0.f;
-  uint64_t inc_S = 1;
+  uint64_t inc_S = 1ull << 52;  // lanes without a step yet form a bracket too: a total in its range (unused)
   bool dead = false;
   auto bracket = [&](uint64_t S) {
     const int e = 63 - __clzll((long long)S);
