@@ -120,17 +120,6 @@ struct StateVec<float, 2> {
   }
 };
 template <>
-struct StateVec<double, 2> {
-  __device__ __forceinline__ static void store(double* X, int j, const double* x) {
-    reinterpret_cast<double2*>(X)[j] = make_double2(x[0], x[1]);
-  }
-  __device__ __forceinline__ static void load(const double* X, int j, double* x) {
-    const double2 v = reinterpret_cast<const double2*>(X)[j];
-    x[0] = v.x;
-    x[1] = v.y;
-  }
-};
-template <>
 struct StateVec<float, 4> {
   __device__ __forceinline__ static void store(float* X, int j, const float* x) {
     reinterpret_cast<float4*>(X)[j] = make_float4(x[0], x[1], x[2], x[3]);
@@ -242,10 +231,9 @@ __device__ __forceinline__ int slots_exact(const SlotCount& sc, uint64_t C, floa
   return n + ((lh < rh || (lh == rh && ll < rl)) ? 1 : 0);
 }
 
-// exp in the working precision: the FP32 path uses the hardware exp2
-// approximation (relative error about 2^-22), the FP64 path the full-precision exp.
+// exp of the FP32 filters: the hardware exp2 approximation (relative error about 2^-22); the FP64
+// filters' exponentials are soft64.cuh's.
 __device__ __forceinline__ float fast_exp(float x) { return __expf(x); }
-__device__ __forceinline__ double fast_exp(double x) { return exp(x); }
 
 // Per-filter constants of the model in the working precision.
 template <typename R, int MODEL>
@@ -737,6 +725,7 @@ __device__ __forceinline__ void run_filter(const PFJob& J, const PFModel& mdl, i
   const int seg = 32 * PPT;  // particles per warp
 
   constexpr bool STAGED = is_staged(PPT);
+  static_assert(STAGED || !F64, "the FP64 filter of up to four particles per thread is run_filter64");
   constexpr bool GEN = GENERAL && !STAGED;
   uint64_t* P = reinterpret_cast<uint64_t*>(region);   // [Mp] inclusive prefix of q (staged, variants)
   R* X = reinterpret_cast<R*>(P + (STAGED || GEN ? Mp : 0));  // [Mp][NS] particle states
