@@ -334,7 +334,10 @@ smc2_status smc2_resample_systematic(const uint64_t* q_dev, int n, uint32_t U, i
  * ctr_dev[4r .. 4r+3] (device), words_dev[4r..] (device, may be NULL)
  * receive Philox4x32-10 of (counter, seed) and z_dev[4r..] (device, may be
  * NULL) the four Box-Muller normals made from them, in double (precision
- * SMC2_PREC_FP64) or float arithmetic widened to double (SMC2_PREC_MIXED). */
+ * SMC2_PREC_FP64) or float arithmetic widened to double (SMC2_PREC_MIXED).
+ * The sampler's proposals and the FP32 filters use these values; the FP64
+ * filters evaluate the same normals in 64-bit integers, within 1.5 ulp of the
+ * exact values, so the two may differ in the last bits. */
 smc2_status smc2_philox_normals(uint64_t seed, const uint32_t* ctr_dev, int n, int precision,
                                 uint32_t* words_dev, double* z_dev, void* stream);
 

@@ -10,8 +10,11 @@
 // followed by a short power series (2^(i/256) and 2^(i/65536) for the exponential;
 // ln of 256 cells for the logarithm; cos and sin at multiples of pi/1024 with the
 // angle-addition formulas; one Halley step for the square root), with every stage
-// carried to 2^-60 or better, so the results are within 0.52 ulp of the exact value
-// (the library's log, exp and sincospi are within 1 ulp).
+// carried to 2^-60 or better.  What that leaves: the exponential is within 2^-56
+// relative before its use, log1p(x) - x next to 0 within half an ulp of x, and a
+// normal within 1.5 ulp (next to a zero of its sine the angle's absolute 2^-64
+// counts; largest seen 1.31 over 6 10^7, root mean square 0.29, 0.7 % beyond
+// 0.52; the library's log and sincospi are within 1 ulp each).
 //
 // Fixed-point notation: "Qk" is an integer holding value 2^k.
 #pragma once
