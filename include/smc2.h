@@ -140,8 +140,13 @@ typedef struct smc2_ctx smc2_ctx; /* opaque; owns its device workspace */
  *   CTA), SMC2_PF_FP32 the register-resident FP32 filter with 2, 4 or 8
  *   particles per thread (mixed precision, LG or SEIR model, the default
  *   filter; one filter per CTA when every dataset's group has the same width,
- *   else groups of unequal width sharing a CTA).  Both compute the same filter;
- *   they differ in speed only.
+ *   else groups of unequal width sharing a CTA).  Both compute the same filter.
+ *   In mixed precision a log-weight's last bits depend on the family and, with
+ *   SMC2_PF_GROUPS, on the launch shape (about 4e-9 relative in a
+ *   log-likelihood; a run then takes another resampling decision now and
+ *   then), and the tuner picks by time: a caller who wants the same bits from
+ *   every context fixes pf_family, and with SMC2_PF_GROUPS ppt and cta_threads
+ *   too.  The FP32 family gives the same bits in all its shapes.
  * n_datasets: number of independent datasets run together (<= 1: one).
  * ds_N, ds_M, ds_T: host arrays of n_datasets sizes (NULL when n_datasets <= 1). */
 typedef struct {
@@ -412,8 +417,8 @@ smc2_status smc2_fma_rates(double* fp32_flops, double* fp64_flops, void* stream)
  * smc2_mlp_adam_step takes them, continuing params, m, v and *step_dev.
  * stdz_dev (device FP64, 2 D + 6 values in the layout of
  * smc2_get_learned_state) receives the standardisation and the loss of the
- * last step before its update (0 when steps = 0).  Allocates a few hundred
- * bytes on `stream` (stream-ordered).  Errors: EINVAL (D outside 1..8, R < 1,
+ * last step before its update (0 when steps = 0).  Allocates nothing.
+ * Errors: EINVAL (D outside 1..8, R < 1,
  * steps outside 0..256, a NULL pointer, params_dev not 16-byte aligned). */
 smc2_status smc2_mlp_loss_grad(int D, const float* params_dev, const float* x_dev, const float* y_dev,
                                int R, float* grad_dev, float* loss_dev, void* stream);

@@ -495,9 +495,10 @@ smc2_status choose_launch_shape(smc2_ctx* c) {
       }
     }
     // The groups kernel's FP32 instantiations for one group per CTA and for several may round a log-weight's
-    // last bit differently (the SIR model's log-likelihoods are 4e-9 apart at ppt 2 with the paper's filter), so
-    // between shapes of the same ppt within the timings' noise, 2 %, the one-group shape is taken: then a tie
-    // does not change results from one context to the next.
+    // last bit differently (the SIR model's log-likelihoods are 4e-9 apart at ppt 2 with the paper's filter).
+    // Between two finalists of the same ppt that differ in this alone and lie within the timings' noise, 2 %,
+    // the one-group shape is taken, so that such a tie does not change results from one context to the next.
+    // Ties between shapes of different ppt or family still fall either way.
     for (size_t f = 0; f < fin.size(); ++f) {
       const Shape &a = cand[fin[f]], &b = cand[pick_i];
       if (c->precision == SMC2_PREC_FP64 || a.fast || b.fast || a.named || !b.named || a.ppt != b.ppt || ts[f].size() < 3) continue;
