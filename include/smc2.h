@@ -28,6 +28,9 @@
  *    hardware barriers) and compute every index they use from exact integer
  *    arithmetic on validated sizes, so no device status exists for an expired
  *    wait or an index out of range.
+ *  - A context reads back through 256 KB of page-locked host memory, which
+ *    smc2_destroy keeps for a later context of the process (16 such buffers at
+ *    most).
  *  - Host threads: calls that read a context (smc2_estimate, smc2_get_history,
  *    smc2_get_proposals, smc2_get_learned_state, smc2_get_learned_training,
  *    smc2_get_state, smc2_sync) may run on several threads at once and beside

@@ -45,6 +45,66 @@ constexpr int kMlpWindow = 4;
 // by itself: 16 us each, 20 of them after a run of 20 iterations).
 constexpr size_t kPinnedBytes = 256 * 1024;
 
+// The buffers of destroyed contexts, kept for the next ones: page-locking and releasing one takes 115 and
+// 170 us, which a program that makes a context for each of its runs would pay every time (LG FP64, N=64/M=128,
+// fixed launch shape: creation 285 us and destruction 238 with a buffer of its own, 174 and 67 with a kept
+// one).  At most 16 are kept, 4 MB in all.  A buffer belongs to the CUDA context that it was made in, and a
+// device reset frees it behind the pool's back: it is handed out only while that very context is current
+// (cuCtxGetId's number is never used again).
+class PinnedPool {
+ public:
+  char* take(unsigned long long id) {
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      for (int i = 0; id != 0 && i < count_; ++i)
+        if (kept_[i].id == id) {
+          char* p = kept_[i].p;
+          kept_[i] = kept_[--count_];
+          return p;
+        }
+    }
+    char* p = nullptr;
+    if (cudaMallocHost(&p, kPinnedBytes) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
+  }
+  void give(char* p, unsigned long long id) {
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      if (id != 0 && count_ < kMax) {
+        kept_[count_++] = {p, id};
+        return;
+      }
+    }
+    cudaFreeHost(p);
+  }
+  // number of the calling thread's current CUDA context; 0 when there is none to be had
+  static unsigned long long context_id() {
+    static const auto get = [] {
+      void* f = nullptr;
+      cudaDriverEntryPointQueryResult found;
+      if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &found) != cudaSuccess) f = nullptr;
+      return reinterpret_cast<int (*)(void*, unsigned long long*)>(f);
+    }();
+    unsigned long long id = 0;
+    return get && get(nullptr, &id) == 0 ? id : 0;
+  }
+
+ private:
+  static constexpr int kMax = 16;
+  struct Kept {
+    char* p;
+    unsigned long long id;
+  };
+  std::mutex mutex_;
+  Kept kept_[kMax] = {};
+  int count_ = 0;
+};
+PinnedPool& pinned_pool() {
+  static PinnedPool& pool = *new PinnedPool;  // outlives every static object that may hold a context
+  return pool;
+}
+
 struct GraphKey {
   int n_iter, timing;
   bool operator<(const GraphKey& o) const {
@@ -84,7 +144,8 @@ struct smc2_ctx {
   int* d_wu_counter = nullptr;
   int* d_k = nullptr;
   int* d_status = nullptr;
-  char* pinned = nullptr;   // page-locked staging of read-backs (kPinnedBytes), held by one read-back at a time
+  char* pinned = nullptr;   // page-locked staging of read-backs (kPinnedBytes), held by one read-back at a time; may be absent
+  unsigned long long pinned_id = 0;
   std::mutex pinned_mutex;
   unsigned* d_grid_ticket = nullptr;
   int ppt = 4, pf_block = 256, pf_grid = 1;
@@ -706,7 +767,7 @@ struct ReadBack {
   int n_pieces = 0;
   size_t used = 16;  // the status word leads the buffer
   explicit ReadBack(smc2_ctx* ctx) : c(ctx), hold(ctx->pinned_mutex) {}
-  static bool fits(size_t bytes, size_t used = 16) { return used + bytes <= kPinnedBytes; }
+  bool fits(size_t bytes) const { return c->pinned && used + bytes <= kPinnedBytes; }
   char* take(size_t bytes) {  // room for a piece that fits
     char* at = c->pinned + used;
     used += (bytes + 15) & ~(size_t)15;
@@ -714,18 +775,19 @@ struct ReadBack {
   }
   cudaError_t add(void* dst, const void* src, size_t bytes) {
     if (!dst || !bytes) return cudaSuccess;
-    if (!fits(bytes, used) || n_pieces == 4)
+    if (!fits(bytes) || n_pieces == 4)
       return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, c->stream);
     char* at = take(bytes);
     pieces[n_pieces++] = {dst, at, bytes};
     return cudaMemcpyAsync(at, src, bytes, cudaMemcpyDeviceToHost, c->stream);
   }
   smc2_status finish() {
-    SMC2_TRY(cudaMemcpyAsync(c->pinned, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    int bits = 0;
+    void* word = c->pinned ? static_cast<void*>(c->pinned) : &bits;
+    SMC2_TRY(cudaMemcpyAsync(word, c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     SMC2_TRY(cudaStreamSynchronize(c->stream));
     for (int i = 0; i < n_pieces; ++i) memcpy(pieces[i].dst, pieces[i].staged, pieces[i].bytes);
-    int bits = 0;
-    memcpy(&bits, c->pinned, sizeof(int));
+    if (c->pinned) memcpy(&bits, c->pinned, sizeof(int));
     return status_from_bits(bits);
   }
 };
@@ -805,7 +867,8 @@ smc2_status smc2_init(const smc2_config* cfg, const double* y, void* stream, smc
       cudaEventCreateWithFlags(&c->ev_tjoin, cudaEventDisableTiming) != cudaSuccess)
     return fail(SMC2_ECUDA);
 
-  if (cudaMallocHost(&c->pinned, kPinnedBytes) != cudaSuccess) return fail(SMC2_ENOMEM);
+  c->pinned_id = PinnedPool::context_id();
+  c->pinned = pinned_pool().take(c->pinned_id);  // absent: read-backs copy straight to the caller
   c->arena_bytes = layout(c, nullptr);
   if (cudaMalloc(&c->arena, c->arena_bytes) != cudaSuccess) return fail(SMC2_ENOMEM);
   layout(c, c->arena);
@@ -951,7 +1014,7 @@ smc2_status smc2_run(smc2_ctx* c, int n_iter, smc2_iter_stats* stats_host) {
   // exceed it in an array that is there before anything runs
   const size_t n_stats = (size_t)c->n_ds * n_iter;
   std::unique_ptr<smc2_iter_stats[]> by_dataset;
-  if (stats_host && c->n_ds > 1 && !ReadBack::fits(n_stats * sizeof(smc2_iter_stats))) {
+  if (stats_host && c->n_ds > 1 && !(c->pinned && 16 + n_stats * sizeof(smc2_iter_stats) <= kPinnedBytes)) {
     by_dataset.reset(new (std::nothrow) smc2_iter_stats[n_stats]);
     if (!by_dataset) return SMC2_ENOMEM;
   }
@@ -1263,7 +1326,7 @@ void smc2_destroy(smc2_ctx* c) {
   if (c->stream || c->arena) cudaStreamSynchronize(c->stream);
   drop_graphs(c);
   if (c->arena) cudaFree(c->arena);
-  if (c->pinned) cudaFreeHost(c->pinned);
+  if (c->pinned) pinned_pool().give(c->pinned, c->pinned_id);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
