@@ -281,7 +281,7 @@ size_t layout(smc2_ctx* c, char* base) {
   char* start = p;
   const int D = c->D;
   c->d_y = carve<double>(p, c->ytot);
-  c->d_k = carve<int>(p, 4);
+  c->d_k = carve<int>(p, 4);  // d_k .. d_wu_counter are cleared together (clear_run_state)
   c->d_status = carve<int>(p, 4);
   c->d_grid_ticket = carve<unsigned>(p, 4);
   c->d_wu_counter = carve<int>(p, 4);
@@ -574,10 +574,8 @@ smc2_status choose_launch_shape(smc2_ctx* c) {
 
 smc2_status clear_run_state(smc2_ctx* c) {
   cudaStream_t s = c->stream;
-  SMC2_TRY(cudaMemsetAsync(c->d_k, 0, 4 * sizeof(int), s));
-  SMC2_TRY(cudaMemsetAsync(c->d_status, 0, 4 * sizeof(int), s));
-  SMC2_TRY(cudaMemsetAsync(c->d_grid_ticket, 0, 4 * sizeof(unsigned), s));
-  SMC2_TRY(cudaMemsetAsync(c->d_wu_counter, 0, 4 * sizeof(int), s));
+  // the iteration counter, the status word, the grid ticket and the queue's counters, neighbours in the arena
+  SMC2_TRY(cudaMemsetAsync(c->d_k, 0, (char*)(c->d_wu_counter + 4) - (char*)c->d_k, s));
   for (int d = 0; d < c->n_ds; ++d) {
     const DSDev& ds = c->h_ds[d];
     SMC2_TRY(cudaMemsetAsync(ds.tickets, 0, 4 * sizeof(unsigned), s));
