@@ -92,7 +92,9 @@ __host__ __device__ inline size_t region_bytes(int Mp, int nw, int ns, int rsize
 }
 
 // Register budget per variant (threads x registers must fit the SM at the
-// shapes the tuner tries); beyond it the compiler spills to local memory.
+// shapes the tuner tries); beyond it the compiler spills to local memory.  The FP64 caps were chosen
+// on the SEIR-type model (see run_filter64); under them the SIR model's filter spills 540 to 1580 bytes
+// at ppt 2 and 4, which has not been weighed against fewer resident warps.
 template <typename R, int PPT>
 struct RegCap {
   static constexpr int value =
@@ -578,7 +580,7 @@ static __device__ __noinline__ double sir_flow_fp64(double n, double p, double h
 // The same model in FP64.  The draws' decisions come from binomial_filtered, whose probability
 // for the S->I flow is 1 - e^(-beta I / npop) in fixed point; draws that it leaves open (one in
 // 8000 at npop = 1e4) run the FP64 sampler, whose results all draws have.
-// N = 256, M = 500, T = 30: 13.8 ms with every draw by the FP64 sampler (FP64 pipe 85 % busy), 0.98 ms so.
+// N = 256, M = 500, T = 30: 13.8 ms with every draw by the FP64 sampler (FP64 pipe 85 % busy), 0.90 ms so.
 template <>
 struct FilterParams<double, MODEL_SIR> {
   double beta, npop, rate, S0, I0, p_ir;  // rate = beta / npop
