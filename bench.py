@@ -68,8 +68,8 @@ MODEL_NAMES = {0: "LG-AR(1)", 1: "SEIR-type", 2: "binomial SIR"}
 # from one ncu capture of a full-size launch of the workload, valid only for that
 # workload and the kernel source it was taken on (sha-256 prefixes of the sources).
 PF_TRAFFIC = {
-    "seir_t200_n8192": {"bytes": 473088.0, "sources": {"pf_fast.cuh": "beb2ebbb6d69873f", "pf_impl.cuh": "8f0fc4af0d014c3f",
-                                                       "common.cuh": "5024364c08332de3"}},
+    "seir_t200_n8192": {"bytes": 464896.0, "sources": {"pf_fast.cuh": "4a689c411e8380be", "pf_impl.cuh": "2e2c6443c89a1cce",
+                                                       "common.cuh": "7a53ecadd2216763"}},
 }
 
 
