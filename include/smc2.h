@@ -264,7 +264,9 @@ smc2_status smc2_iterate(smc2_ctx* ctx, smc2_iter_stats* stats_host);
 /* n_iter iterations back to back without host synchronisation (captured
  * once as a CUDA graph and replayed).  stats_host (may be NULL) receives
  * n_iter * n_datasets entries, iteration-major, and makes the call
- * synchronise.  Errors: ESTATE when fewer than n_iter iterations remain. */
+ * synchronise.  Errors: ESTATE when fewer than n_iter iterations remain,
+ * ENOMEM when no host memory is left for the statistics of many datasets
+ * (nothing has run then). */
 smc2_status smc2_run(smc2_ctx* ctx, int n_iter, smc2_iter_stats* stats_host);
 
 /* Recycled estimate after the iterations run so far (Sec. IV-C, Eq. 29 with
